@@ -179,17 +179,31 @@ PoissonPlan::~PoissonPlan()
 
 namespace {
 
-__global__ void k_twiddles(int M, void *out, int dbl)
+// Entry i of a length's table: exp(-2 pi i exps[i] / M).
+__global__ void k_twiddles(int M, const int *__restrict__ exps, void *out, int dbl)
 {
-    const int m = blockIdx.x * blockDim.x + threadIdx.x;
-    if (m >= M) return;
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= M) return;
     double s, c;
-    sincospi(-2.0 * m / M, &s, &c);
+    sincospi(-2.0 * exps[i] / M, &s, &c);
     if (dbl) {
-        ((Cx<double> *)out)[m] = {c, s};
+        ((Cx<double> *)out)[i] = {c, s};
     } else {
-        ((Cx<float> *)out)[m] = {(float)c, (float)s};
+        ((Cx<float> *)out)[i] = {(float)c, (float)s};
     }
+}
+
+// The table's exponents in the order of the length's stage plan.
+template <int ML>
+lgf_status fill_exponents(std::vector<int> *e)
+{
+    for (int i = 0; i < ML; ++i) (*e)[i] = pk::twiddle_exponent<ML>(i);
+    return LGF_OK;
+}
+lgf_status twiddle_exponents(lgf_ctx *ctx, int M, std::vector<int> *e)
+{
+    e->assign(M, 0);
+    LGF_DISPATCH_ML(M, fill_exponents<LM>(e));
 }
 
 // Spectrum of a shifted window: the complex forward transform at
@@ -347,14 +361,23 @@ const void *twiddles(lgf_ctx *ctx, int M, bool dbl, lgf_status *st)
     auto &tab = dbl ? ctx->tw64 : ctx->tw32;
     auto it = tab.find(M);
     if (it != tab.end()) return it->second;
+    std::vector<int> exps;
+    if ((*st = twiddle_exponents(ctx, M, &exps)) != LGF_OK) return nullptr;
     void *p = nullptr;
+    int *ed = nullptr;
     cudaError_t e = cudaMalloc(&p, (size_t)M * (dbl ? 16 : 8));
+    if (e == cudaSuccess) e = cudaMalloc(&ed, (size_t)M * sizeof(int));
     if (e != cudaSuccess) {
+        cudaFree(p);
         *st = fail(ctx, LGF_ENOMEM, "twiddle table allocation failed");
         return nullptr;
     }
-    k_twiddles<<<(M + 255) / 256, 256>>>(M, p, dbl ? 1 : 0);
-    e = cudaDeviceSynchronize();
+    e = cudaMemcpy(ed, exps.data(), (size_t)M * sizeof(int), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) {
+        k_twiddles<<<(M + 255) / 256, 256>>>(M, ed, p, dbl ? 1 : 0);
+        e = cudaDeviceSynchronize();
+    }
+    cudaFree(ed);
     if (e != cudaSuccess) {
         cudaFree(p);
         *st = cuda_fail(ctx, e, "twiddle kernel");

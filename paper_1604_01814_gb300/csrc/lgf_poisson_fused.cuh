@@ -143,9 +143,9 @@ __global__ void __cluster_dims__(NCL, 1, 1) __launch_bounds__(YXCfg<MY, MX>::THR
 #pragma unroll
                     for (int q = 0; q < R0; ++q) a[q] = s[ad(w, q * PY::G0 + gg)];
                     if (half)
-                        dit_group<R0, 1, true>(a, gg, tw);
+                        dit_group<R0, PY::G0, true>(a, gg, tw);
                     else
-                        dit_group<R0, 1, false>(a, gg, tw);
+                        dit_group<R0, PY::G0, false>(a, gg, tw);
                     if (live) {
                         const int r = gg - lo;
 #pragma unroll

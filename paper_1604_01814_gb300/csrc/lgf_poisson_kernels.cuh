@@ -49,6 +49,7 @@ struct Plan {
     static constexpr int N1 = M / R0;                             // sub-problem size entering stage 1
     static constexpr int G0 = M / R0, G1 = M / R1, GL = M / RL;   // groups per stage
     static constexpr int TPC = cgcd(cgcd(G0, NST == 3 ? G1 : G0), GL);
+    static constexpr int TW1 = (R0 - 1) * G0;                     // first twiddle of the middle stage
     static_assert(R0 * R1 * RL == M && RL <= 20 && RL >= 4, "plan must cover the length");
     static_assert(G0 % TPC == 0 && G1 % TPC == 0 && GL % TPC == 0, "whole groups per thread");
 };
@@ -66,6 +67,27 @@ __device__ __forceinline__ int pos_of(int k)
     return q0 * (ML / P::R0) + q1 * P::RL + qL;
 }
 
+// The column passes are bound by instruction issue (76 % of the slots of the z
+// pass at length 320), and more than a quarter of their instructions were index
+// arithmetic: twiddles gathered at j q M/N from one natural-order table, a division
+// per middle-stage group, 64-bit offsets formed per access.  Tables in the order
+// of the stages, a middle stage that splits each line as sub-problems times groups
+// and pointers that walk took the refresh of 556 blocks (x 640, y and z 320) from
+// 826 to 730 us, the 64-plate batch from 4.85 to 4.42 ms and the 512x256x256 wake
+// from 7.39 to 6.90 ms, every output bit the same; the x passes also lost the bank
+// conflicts of the gathered twiddles.
+// Exponent e of entry i of a length's twiddle table (the entry is
+// exp(-2 pi i e / M)): the first stage's w_M^{j q} at (q - 1) G0 + j, then the
+// middle stage's w_{N1}^{j q} = w_M^{j q R0} at TW1 + (q - 1) RL + j; 0 past them.
+template <int ML>
+int twiddle_exponent(int i)
+{
+    using P = Plan<ML>;
+    if (i < P::TW1) return (i % P::G0) * (i / P::G0 + 1);
+    i -= P::TW1;
+    return P::NST == 3 && i < (P::R1 - 1) * P::RL ? (i % P::RL) * (i / P::RL + 1) * P::R0 : 0;
+}
+
 template <int ML>
 __device__ __forceinline__ int freq_of(int pos)
 {
@@ -76,9 +98,11 @@ __device__ __forceinline__ int freq_of(int pos)
 }
 
 // Forward butterfly of one group of a stage that is not the last: DFT then
-// twiddles w_N^{j q} = tw[j q TWS] (TWS = M/N).  HALF: the inputs
-// a[R/2..R) are zero (not read).
-template <int R, int TWS, bool HALF = false, typename T>
+// the twiddles w_N^{j q}, which the table holds at tw[(q - 1) J + j] for the
+// stage's J groups (see twiddle_exponent), so that one address per thread
+// and constant offsets reach all of them.  HALF: the inputs a[R/2..R) are zero
+// (not read).
+template <int R, int J, bool HALF = false, typename T>
 __device__ __forceinline__ void dif_group(Cx<T> *a, int j, const Cx<T> *tw)
 {
     if constexpr (HALF)
@@ -86,53 +110,62 @@ __device__ __forceinline__ void dif_group(Cx<T> *a, int j, const Cx<T> *tw)
     else
         Dft<R, -1, T>::run(a);
 #pragma unroll
-    for (int q = 1; q < R; ++q) a[q] = cmul(a[q], tw[j * q * TWS]);
+    for (int q = 1; q < R; ++q) a[q] = cmul(a[q], tw[(q - 1) * J + j]);
 }
 
 // A group whose only nonzero input is a[0] (the data of the line end before
 // M/R): the DFT gives a[0] at every output, so the stage is the twiddles.
-template <int R, int TWS, typename T>
+template <int R, int J, typename T>
 __device__ __forceinline__ void dif_group_single(Cx<T> *a, int j, const Cx<T> *tw)
 {
 #pragma unroll
-    for (int q = 1; q < R; ++q) a[q] = cmul(a[0], tw[j * q * TWS]);
+    for (int q = 1; q < R; ++q) a[q] = cmul(a[0], tw[(q - 1) * J + j]);
 }
 
 // Its adjoint.  HALF: only the outputs a[0..R/2) are formed.
-template <int R, int TWS, bool HALF = false, typename T>
+template <int R, int J, bool HALF = false, typename T>
 __device__ __forceinline__ void dit_group(Cx<T> *a, int j, const Cx<T> *tw)
 {
 #pragma unroll
-    for (int q = 1; q < R; ++q) a[q] = cmulc(a[q], tw[j * q * TWS]);
+    for (int q = 1; q < R; ++q) a[q] = cmulc(a[q], tw[(q - 1) * J + j]);
     if constexpr (HALF)
         dft_half_out<R, 1, T>(a);
     else
         Dft<R, 1, T>::run(a);
 }
 
-// Middle stage (three-stage plans): shared memory to shared memory.
+// Middle stage (three-stage plans): shared memory to shared memory.  The
+// threads of a line split as TS sub-problems times TJ groups, so that every
+// group's address is the thread's own plus a constant.
 template <int ML, int DIR, typename T, class Addr>
 __device__ __forceinline__ void middle_stage(Cx<T> *s, const Addr &ad, int line, int t, const Cx<T> *tw)
 {
     using P = Plan<ML>;
     if constexpr (P::NST == 3) {
         constexpr int N = P::N1, R = P::R1, NP = N / R;
+        constexpr int TS = cgcd(P::TPC, P::R0), TJ = P::TPC / TS;
+        static_assert(NP % TJ == 0, "whole groups per thread");
+        const int j0 = t / TS;
+        const Cx<T> *tw1 = tw + P::TW1 + j0;
+        const int o = (t % TS) * N + j0;
 #pragma unroll
-        for (int g = t; g < P::G1; g += P::TPC) {
-            const int sub = g / NP, j = g % NP, o = sub * N;
-            Cx<T> a[R];
-            if (DIR < 0) {
+        for (int sub = 0; sub < P::R0; sub += TS) {
 #pragma unroll
-                for (int p = 0; p < R; ++p) a[p] = s[ad(line, o + j + p * NP)];
-                dif_group<R, P::R0>(a, j, tw);
+            for (int j = 0; j < NP; j += TJ) {
+                Cx<T> a[R];
+                if (DIR < 0) {
 #pragma unroll
-                for (int q = 0; q < R; ++q) s[ad(line, o + q * NP + j)] = a[q];
-            } else {
+                    for (int p = 0; p < R; ++p) a[p] = s[ad(line, o + sub * N + j + p * NP)];
+                    dif_group<R, NP>(a, j, tw1);
 #pragma unroll
-                for (int q = 0; q < R; ++q) a[q] = s[ad(line, o + q * NP + j)];
-                dit_group<R, P::R0>(a, j, tw);
+                    for (int q = 0; q < R; ++q) s[ad(line, o + sub * N + q * NP + j)] = a[q];
+                } else {
 #pragma unroll
-                for (int p = 0; p < R; ++p) s[ad(line, o + j + p * NP)] = a[p];
+                    for (int q = 0; q < R; ++q) a[q] = s[ad(line, o + sub * N + q * NP + j)];
+                    dit_group<R, NP>(a, j, tw1);
+#pragma unroll
+                    for (int p = 0; p < R; ++p) s[ad(line, o + sub * N + j + p * NP)] = a[p];
+                }
             }
         }
     }
@@ -274,12 +307,12 @@ __device__ __forceinline__ void col_forward_body(int bx, int by, const Cx<T> *__
 #pragma unroll
         for (int i = 0; i < NG0; ++i) {
             const int r = t + i * P::TPC - lo;   // data row of digit p = 0
-            int64_t off = (int64_t)r * rs;
+            const Cx<T> *src = ib + (int64_t)r * rs;
 #pragma unroll
             for (int p = 0; p < NP; ++p) {
                 const bool ok = live && (unsigned)(r + p * P::G0) < (unsigned)n;
-                a[i][p] = ok ? ib[off] : Cx<T>{T(0), T(0)};
-                off += istep;
+                a[i][p] = ok ? *src : Cx<T>{T(0), T(0)};
+                src += istep;
             }
         }
     } else {
@@ -287,13 +320,13 @@ __device__ __forceinline__ void col_forward_body(int bx, int by, const Cx<T> *__
 #pragma unroll
         for (int i = 0; i < NG0; ++i) {
             const int r = t + i * P::TPC - lo;
-            int64_t off = (int64_t)r * rs;
+            const Cx<T> *src = ib + (int64_t)r * rs;
 #pragma unroll
             for (int p = 0; p < NP; ++p) {
                 const int y = r + p * P::G0;
                 const bool ok = live && (unsigned)y < (unsigned)n && rf.row(pm, y);
-                a[i][p] = ok ? ib[off] : Cx<T>{T(0), T(0)};
-                off += istep;
+                a[i][p] = ok ? *src : Cx<T>{T(0), T(0)};
+                src += istep;
             }
         }
     }
@@ -301,7 +334,7 @@ __device__ __forceinline__ void col_forward_body(int bx, int by, const Cx<T> *__
 #pragma unroll
     for (int i = 0; i < NG0; ++i) {
         const int g = t + i * P::TPC;
-        dif_group<P::R0, 1, HALF>(a[i], g, tw);
+        dif_group<P::R0, P::G0, HALF>(a[i], g, tw);
 #pragma unroll
         for (int q = 0; q < R0; ++q) s[ad(w, q * P::G0 + g)] = a[i][q];
     }
@@ -319,11 +352,11 @@ __device__ __forceinline__ void col_forward_body(int bx, int by, const Cx<T> *__
         for (int q = 0; q < RL; ++q) c[q] = s[ad(w, (g * P::RL) + q)];
         Dft<RL, -1, T>::run(c);
         if (live) {
-            int64_t off = (int64_t)freq_of<ML>(g * P::RL) * os;
+            Cx<T> *dst = ob + (int64_t)freq_of<ML>(g * P::RL) * os;
 #pragma unroll
             for (int q = 0; q < RL; ++q) {
-                ob[off] = c[q];
-                off += ostep;
+                *dst = c[q];
+                dst += ostep;
             }
         }
     }
@@ -370,11 +403,11 @@ __device__ __forceinline__ void col_inverse_body(int bx, int by, const Cx<T> *__
 #pragma unroll
     for (int i = 0; i < NGL; ++i) {
         const int g = t + i * P::TPC;
-        int64_t off = (int64_t)freq_of<ML>(g * P::RL) * rs;
+        const Cx<T> *src = ib + (int64_t)freq_of<ML>(g * P::RL) * rs;
 #pragma unroll
         for (int q = 0; q < RL; ++q) {
-            c[i][q] = live ? ib[off] : Cx<T>{T(0), T(0)};
-            off += istep;
+            c[i][q] = live ? *src : Cx<T>{T(0), T(0)};
+            src += istep;
         }
     }
 #pragma unroll
@@ -397,14 +430,14 @@ __device__ __forceinline__ void col_inverse_body(int bx, int by, const Cx<T> *__
         Cx<T> a[R0];
 #pragma unroll
         for (int q = 0; q < R0; ++q) a[q] = s[ad(w, q * P::G0 + g)];
-        dit_group<P::R0, 1, HALF_OUT>(a, g, tw);
+        dit_group<P::R0, P::G0, HALF_OUT>(a, g, tw);
         if (live) {
             const int r = g - lo;
-            int64_t off = (int64_t)r * os;
+            Cx<T> *dst = ob + (int64_t)r * os;
 #pragma unroll
             for (int p = 0; p < NOUT; ++p) {
-                if ((unsigned)(r + p * P::G0) < (unsigned)n) ob[off] = a[p];
-                off += ostep;
+                if ((unsigned)(r + p * P::G0) < (unsigned)n) *dst = a[p];
+                dst += ostep;
             }
         }
     }
@@ -472,19 +505,19 @@ __device__ __forceinline__ void col_convolve_body(int bx, int nf, Cx<T> *__restr
 #pragma unroll
         for (int i = 0; i < NG0; ++i) {
             const int r = t + i * P::TPC - s0;
-            int64_t off = (int64_t)r * plane;
+            const Cx<T> *src = bb + (int64_t)r * plane;
 #pragma unroll
             for (int p = 0; p < R0 / 2; ++p) {
                 const bool ok = live && (unsigned)(r + p * P::G0) < (unsigned)ns;
-                a[i][p] = ok ? bb[off] : Cx<T>{T(0), T(0)};
-                off += step0;
+                a[i][p] = ok ? *src : Cx<T>{T(0), T(0)};
+                src += step0;
             }
         }
         __syncthreads();
 #pragma unroll
         for (int i = 0; i < NG0; ++i) {
             const int g = t + i * P::TPC;
-            dif_group<P::R0, 1, true>(a[i], g, tw);
+            dif_group<P::R0, P::G0, true>(a[i], g, tw);
 #pragma unroll
             for (int q = 0; q < R0; ++q) s[ad(w, q * P::G0 + g)] = a[i][q];
         }
@@ -499,20 +532,24 @@ __device__ __forceinline__ void col_convolve_body(int bx, int nf, Cx<T> *__restr
     const int Khy = SPEC == 2 ? My : My / 2 + 1;
     const int kyr = SPEC == 2 ? ky : (ky <= My - ky ? ky : My - ky);
     const SpecT *sp = spec + (int64_t)kyr * K + kx;
-    const int64_t sp_plane = (int64_t)Khy * K;
+    const int64_t sp_plane = (int64_t)Khy * K, sp_step = S * sp_plane;
 #pragma unroll
     for (int g = t; g < P::GL; g += P::TPC) {
         // frequency of digit q: kb + q S; its mirror M - kb - q S once past M/2
         const int kb = freq_of<ML>(g * P::RL);
         const SpecT *spl = sp + (int64_t)kb * sp_plane;
-        const SpecT *sph = sp + (int64_t)(M - kb) * sp_plane;
+        const SpecT *sph = sp + (int64_t)(M - kb - (RL / 2) * S) * sp_plane;
         Cx<T> c[RL];
         SpecT gk[RL];
 #pragma unroll
-        for (int q = 0; q < RL; ++q) {
-            gk[q] = q < RL / 2 ? spl[(int64_t)(q * S) * sp_plane] : sph[-(int64_t)(q * S) * sp_plane];
-            c[q] = s[ad(w, (g * P::RL) + q)];
+        for (int q = 0; q < RL / 2; ++q) {
+            gk[q] = *spl;
+            gk[RL / 2 + q] = *sph;
+            spl += sp_step;
+            sph -= sp_step;
         }
+#pragma unroll
+        for (int q = 0; q < RL; ++q) c[q] = s[ad(w, (g * P::RL) + q)];
         Dft<RL, -1, T>::run(c);
 #pragma unroll
         for (int q = 0; q < RL; ++q) {
@@ -538,14 +575,14 @@ __device__ __forceinline__ void col_convolve_body(int bx, int nf, Cx<T> *__restr
         Cx<T> a[R0];
 #pragma unroll
         for (int q = 0; q < R0; ++q) a[q] = s[ad(w, q * P::G0 + g)];
-        dit_group<P::R0, 1, true>(a, g, tw);
+        dit_group<P::R0, P::G0, true>(a, g, tw);
         if (live) {
             const int r = g - t0;
-            int64_t off = (int64_t)r * plane;
+            Cx<T> *dst = bb + (int64_t)r * plane;
 #pragma unroll
             for (int p = 0; p < R0 / 2; ++p) {
-                if ((unsigned)(r + p * P::G0) < (unsigned)nt) bb[off] = a[p];
-                off += step1;
+                if ((unsigned)(r + p * P::G0) < (unsigned)nt) *dst = a[p];
+                dst += step1;
             }
         }
     }
@@ -640,9 +677,9 @@ __device__ __forceinline__ void row_forward_body(int bx, int by, const T *__rest
     for (int i = 0; i < NG0; ++i) {
         const int gg = t + i * P::TPC;
         if (single)
-            dif_group_single<P::R0, 1>(a[i], gg, tw);
+            dif_group_single<P::R0, P::G0>(a[i], gg, tw);
         else
-            dif_group<P::R0, 1, HALF>(a[i], gg, tw);
+            dif_group<P::R0, P::G0, HALF>(a[i], gg, tw);
 #pragma unroll
         for (int q = 0; q < R0; ++q) s[ad(l, q * P::G0 + gg)] = a[i][q];
     }
@@ -780,7 +817,7 @@ __device__ __forceinline__ void row_inverse_line(int t, int l, bool live, int zi
         Cx<T> a[R0];
 #pragma unroll
         for (int q = 0; q < R0; ++q) a[q] = s[ad(l, q * P::G0 + gg)];
-        dit_group<P::R0, 1, HALF_OUT>(a, gg, tw);
+        dit_group<P::R0, P::G0, HALF_OUT>(a, gg, tw);
         const int xr = gg - g.t0[0];
 #pragma unroll
         for (int p = 0; p < NOUT; ++p) {

@@ -258,3 +258,22 @@ def test_shifted_window_every_point(prec, case, ctx64, ctx32, oracle):
     got = run_poisson(ctx, p)
     ref = oracle_fields(oracle, p)
     assert rel_linf(got, ref) < TOL[prec]
+
+
+FFT_SIZES = (32, 64, 80, 96, 128, 160, 192, 256, 320, 384, 512, 640, 768, 1024, 1280, 1536, 2048, 2560, 3072, 4096)
+
+
+@pytest.mark.parametrize("prec", ["f64", "f32"])
+@pytest.mark.parametrize("axis", [0, 1, 2])
+@pytest.mark.parametrize("M", FFT_SIZES)
+def test_every_transform_length(M, axis, prec, ctx64, ctx32, oracle):
+    """Each stage plan along each axis: blocks at the ends and in the middle
+    of the longest extent that the length embeds."""
+    ctx = ctx64 if prec == "f64" else ctx32
+    b, last = 8, M // 16 - 1
+    c = np.zeros((3, 3), dtype=np.int32)
+    c[:, axis] = (0, last // 2, last)
+    c = np.unique(c, axis=0)
+    f = np.random.default_rng(M + axis).uniform(-1, 1, (1, 1, c.shape[0], b ** 3))
+    p = li.Problem("line", b, c, c.copy(), f)
+    assert rel_linf(run_poisson(ctx, p), oracle_fields(oracle, p)) < TOL[prec]
