@@ -516,18 +516,20 @@ lgf_status lgf_nested_projection_stage(lgf_ctx *ctx, const lgf_stage *st, void *
     IBPlan *pib = nullptr;
     if (nm > 0 && (rc = ib_plan(ctx, D, &pib)) != LGF_OK) return rc;
     // stage buffers: q (cells of D), dd (cells of Dm), v, w, g (faces of D),
-    // U, rhs, y, fh (3 nm each), each 256-byte aligned
+    // U, rhs, y, fh (3 nm each), the force solve's partial sums, each 256-byte
+    // aligned
     const size_t esz = elem_size(ctx);
     auto al = [](size_t n) { return (n + 255) & ~size_t(255); };
     const size_t n_q = al(nD * b3 * esz), n_d = al(Dm.nblocks * b3 * esz), n_v = al(3 * nD * b3 * esz),
                  n_m = al((size_t)3 * nm * esz + 1);
     Scratch &sc = ctx->scr[0];
-    if ((rc = ensure_scratch(ctx, &sc.G, &sc.g, n_q + n_d + 3 * n_v + 4 * n_m)) != LGF_OK) return rc;
+    const size_t n_p = nm > 0 ? stage_force_scratch(ctx, st->W2_dev, (int)(3 * nm)) : 0;
+    if ((rc = ensure_scratch(ctx, &sc.G, &sc.g, n_q + n_d + 3 * n_v + 4 * n_m + n_p)) != LGF_OK) return rc;
     unsigned char *base = (unsigned char *)sc.G;
     void *q = base, *dd = base + n_q, *v = base + n_q + n_d, *w = base + n_q + n_d + n_v,
          *g = base + n_q + n_d + 2 * n_v;
     unsigned char *mk = base + n_q + n_d + 3 * n_v;
-    void *U = mk, *rhs = mk + n_m, *y = mk + 2 * n_m, *fh = mk + 3 * n_m;
+    void *U = mk, *rhs = mk + n_m, *y = mk + 2 * n_m, *fh = mk + 3 * n_m, *part = mk + 4 * n_m;
     const double dx = st->dx;
     // ip (Eq. nested_proj-ip): L_C d* = -G^dagger r = Dbar r
     if ((rc = stage_div(ctx, pdiv, st->r_dev, nullptr, q, dx, s)) != LGF_OK) return rc;
@@ -538,7 +540,8 @@ lgf_status lgf_nested_projection_stage(lgf_ctx *ctx, const lgf_stage *st, void *
         if ((rc = stage_grad(ctx, pgrad, dd, st->r_dev, nullptr, v, dx, s)) != LGF_OK) return rc;
         if ((rc = intf_run(ctx, pi.plan, pi.w, v, w, 3, s)) != LGF_OK) return rc;
         if ((rc = ib_run(ctx, pib, false, nm, st->X_dev, w, U, 1, 1.0, s)) != LGF_OK) return rc;
-        if ((rc = stage_force(ctx, U, st->ub_dev, st->W1_dev, st->W2_dev, rhs, y, fh, (int)(3 * nm), s)) != LGF_OK)
+        if ((rc = stage_force(ctx, U, st->ub_dev, st->W1_dev, st->W2_dev, rhs, y, fh, part, (int)(3 * nm), s)) !=
+            LGF_OK)
             return rc;
         // (I^{i-1})^dagger f_hat = dx^3 R f_hat: the bare kernel sum (R at dx = 1)
         if ((rc = ib_run(ctx, pib, true, nm, st->X_prev_dev, fh, g, 1, 1.0, s)) != LGF_OK) return rc;

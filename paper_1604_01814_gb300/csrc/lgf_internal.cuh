@@ -360,8 +360,10 @@ lgf_status stage_div(lgf_ctx *ctx, const CurlPlan *pl, const void *a, const void
                      cudaStream_t s);
 lgf_status stage_grad(lgf_ctx *ctx, const CurlPlan *pl, const void *d, const void *a, const void *c, void *out,
                       double dx, cudaStream_t s);
+// Bytes of stage_force's `part` buffer for vectors of n values (0: not used).
+size_t stage_force_scratch(const lgf_ctx *ctx, const void *W2, int n);
 lgf_status stage_force(lgf_ctx *ctx, const void *U, const void *ub, const void *W1, const void *W2, void *rhs, void *y,
-                       void *fh, int n, cudaStream_t s);
+                       void *fh, void *part, int n, cudaStream_t s);
 
 // Immersed-boundary operators (lgf_ib.cu)
 lgf_status ib_plan(lgf_ctx *ctx, const lgf_blockset *set, IBPlan **out);

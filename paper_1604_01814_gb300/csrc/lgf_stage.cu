@@ -10,6 +10,9 @@
 // and G^dagger = -Dbar.  Both read the block itself and, where the shift
 // leaves it, the neighbour block of a CurlPlan (dir +1 for Dbar, -1 for G);
 // values outside the input block set are zero.  One thread per output cell.
+#include <algorithm>
+#include <cstring>
+
 #include "lgf_async.cuh"
 #include "lgf_internal.cuh"
 
@@ -125,6 +128,163 @@ __global__ void __launch_bounds__(256) k_gemv_t(const T *__restrict__ W, const T
     }
 }
 
+// f = W^T (W x), x = U - ub, in one pass over W (n x n, row-major), which the
+// two products read once each: HBM bounds both (15360^2 in FP32 is 944 MB, 139
+// us at the measured copy bandwidth).  A CTA of 512 threads holds a whole row
+// in registers (NK 16-byte vectors per thread, the vectors of a warp
+// contiguous), forms y_r = W_r x, and adds y_r W_r to its own sum of W^T y, also in
+// registers; the next row is in flight meanwhile.  One barrier per row (the
+// partial sums of the warps alternate between two buffers).  CTA g's sum goes to
+// part[g], added in a fixed order by k_part_sum.  Rows go round robin to one
+// CTA per SM.  VEC: 16-byte loads (n a multiple of the vector, W aligned).
+constexpr int kGramThreads = 512;
+template <typename T>
+struct GramVec;
+template <>
+struct GramVec<float> {
+    using V = float4;
+};
+template <>
+struct GramVec<double> {
+    using V = double2;
+};
+template <typename T, int NK, bool VEC>
+__global__ void __launch_bounds__(kGramThreads, 1) k_gram(const T *__restrict__ W, const T *__restrict__ U,
+                                                          const T *__restrict__ ub, T *__restrict__ part, int n)
+{
+    using VT = typename GramVec<T>::V;
+    constexpr int NV = sizeof(VT) / sizeof(T), NT = kGramThreads, NW = NT / 32;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    T *xs = reinterpret_cast<T *>(smem_raw);   // [NK * NT * NV], zero past n
+    __shared__ T red[2][NW];
+    const int tid = threadIdx.x;
+    for (int i = tid; i < NK * NT * NV; i += NT) xs[i] = i < n ? U[i] - ub[i] : T(0);
+    __syncthreads();
+    auto load = [&](T (&a)[NK][NV], int row) {
+        const T *w = W + (int64_t)row * n;
+#pragma unroll
+        for (int k = 0; k < NK; ++k) {
+            const int c = (k * NT + tid) * NV;
+            if constexpr (VEC) {
+                const VT v = c < n ? __ldcs(reinterpret_cast<const VT *>(w + c)) : VT{};
+                memcpy(a[k], &v, sizeof(VT));
+            } else {
+#pragma unroll
+                for (int e = 0; e < NV; ++e) a[k][e] = c + e < n ? w[c + e] : T(0);
+            }
+        }
+    };
+    T acc[NK][NV], cur[NK][NV], nxt[NK][NV];
+#pragma unroll
+    for (int k = 0; k < NK; ++k)
+#pragma unroll
+        for (int e = 0; e < NV; ++e) acc[k][e] = T(0);
+    auto row_step = [&](const T (&a)[NK][NV], int buf) {
+        T s = T(0);
+#pragma unroll
+        for (int k = 0; k < NK; ++k) {
+            const VT xv = *reinterpret_cast<const VT *>(xs + (k * NT + tid) * NV);
+            const T *x = reinterpret_cast<const T *>(&xv);
+#pragma unroll
+            for (int e = 0; e < NV; ++e) s += a[k][e] * x[e];
+        }
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+        if ((tid & 31) == 0) red[buf][tid >> 5] = s;
+        __syncthreads();
+        T y = T(0);
+#pragma unroll
+        for (int q = 0; q < NW; ++q) y += red[buf][q];
+#pragma unroll
+        for (int k = 0; k < NK; ++k)
+#pragma unroll
+            for (int e = 0; e < NV; ++e) acc[k][e] += y * a[k][e];
+    };
+    const int g = gridDim.x;
+    int r = blockIdx.x;   // gridDim.x <= n
+    load(cur, r);
+    for (; r < n; r += 2 * g) {
+        if (r + g < n) load(nxt, r + g);
+        row_step(cur, 0);
+        if (r + g >= n) break;   // uniform over the CTA
+        if (r + 2 * g < n) load(cur, r + 2 * g);
+        row_step(nxt, 1);
+    }
+    T *o = part + (int64_t)blockIdx.x * n;
+#pragma unroll
+    for (int k = 0; k < NK; ++k) {
+        const int c = (k * NT + tid) * NV;
+#pragma unroll
+        for (int e = 0; e < NV; ++e)
+            if (c + e < n) o[c + e] = acc[k][e];
+    }
+}
+
+// y = sum of the m rows of part (m x n): k_gemv_t's split with unit weights.
+template <typename T>
+__global__ void __launch_bounds__(256) k_part_sum(const T *__restrict__ part, T *__restrict__ y, int m, int n)
+{
+    __shared__ T sum[8][32];
+    const int col = blockIdx.x * 32 + (threadIdx.x & 31);
+    const int g = threadIdx.x >> 5;
+    T s = T(0);
+    if (col < n)
+        for (int i = g; i < m; i += 8) s += part[(int64_t)i * n + col];
+    sum[g][threadIdx.x & 31] = s;
+    __syncthreads();
+    if (g == 0 && col < n) {
+        T t = T(0);
+#pragma unroll
+        for (int q = 0; q < 8; ++q) t += sum[q][threadIdx.x];
+        y[col] = t;
+    }
+}
+
+template <typename T, int NK, bool VEC>
+lgf_status launch_gram_k(lgf_ctx *ctx, const T *W, const T *U, const T *ub, T *part, T *fh, int n, int grid,
+                         cudaStream_t s)
+{
+    constexpr size_t smem = (size_t)NK * kGramThreads * 16;
+    auto kern = k_gram<T, NK, VEC>;
+    if (smem > 48 * 1024) {
+        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return cuda_fail(ctx, e, "cudaFuncSetAttribute");
+    }
+    kern<<<grid, kGramThreads, smem, s>>>(W, U, ub, part, n);
+    k_part_sum<T><<<(n + 31) / 32, 256, 0, s>>>(part, fh, grid, n);
+    return LGF_OK;
+}
+
+// The row length a thread's NK vectors cover picks NK: 1, 2, 4 or 8.
+template <typename T, bool VEC>
+lgf_status launch_gram(lgf_ctx *ctx, const T *W, const T *U, const T *ub, T *part, T *fh, int n, int grid,
+                       cudaStream_t s)
+{
+    constexpr int per = kGramThreads * (16 / (int)sizeof(T));
+    if (n <= per) return launch_gram_k<T, 1, VEC>(ctx, W, U, ub, part, fh, n, grid, s);
+    if (n <= 2 * per) return launch_gram_k<T, 2, VEC>(ctx, W, U, ub, part, fh, n, grid, s);
+    if (n <= 4 * per) return launch_gram_k<T, 4, VEC>(ctx, W, U, ub, part, fh, n, grid, s);
+    return launch_gram_k<T, 8, VEC>(ctx, W, U, ub, part, fh, n, grid, s);
+}
+
+template <typename T>
+lgf_status gram(lgf_ctx *ctx, const void *W, const void *U, const void *ub, void *part, void *fh, int n, int grid,
+                cudaStream_t s)
+{
+    const bool vec = n % (16 / (int)sizeof(T)) == 0 && reinterpret_cast<uintptr_t>(W) % 16 == 0;
+    return vec ? launch_gram<T, true>(ctx, (const T *)W, (const T *)U, (const T *)ub, (T *)part, (T *)fh, n, grid, s)
+               : launch_gram<T, false>(ctx, (const T *)W, (const T *)U, (const T *)ub, (T *)part, (T *)fh, n, grid, s);
+}
+
+// CTAs of the one-pass product (0: rows too long for a CTA's registers).
+int gram_grid(const lgf_ctx *ctx, int n)
+{
+    const int most = 8 * kGramThreads * (ctx->prec == LGF_F64 ? 2 : 4);   // 16384 in FP32, 8192 in FP64
+    int nsm = 0;
+    if (n > most || cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, ctx->device) != cudaSuccess) return 0;
+    return std::min(n, nsm);
+}
+
 template <typename T, int LB>
 void launch_div_lb(dim3 grid, cudaStream_t s, const T *a, const T *c, T *out, const int *nbr, int64_t ncell,
                    int64_t in_c, T scale)
@@ -234,11 +394,28 @@ lgf_status wait_selftest(lgf_ctx *ctx, long long cycles, cudaStream_t s)
     return LGF_OK;
 }
 
+size_t stage_force_scratch(const lgf_ctx *ctx, const void *W2, int n)
+{
+    return W2 ? 0 : (size_t)gram_grid(ctx, n) * n * (ctx->prec == LGF_F64 ? 8 : 4);
+}
+
 // rhs = U - ub; y = W1 rhs; fh = W2 y (W2 null: W1^T y).  Vectors of n values.
+// W2 null and rows that fit a CTA's registers: both products in one pass over
+// W1 (k_gram; part as sized by stage_force_scratch, rhs and y unused).  On
+// 15360^2 FP32 the two products took 450 us.
 lgf_status stage_force(lgf_ctx *ctx, const void *U, const void *ub, const void *W1, const void *W2, void *rhs, void *y,
-                       void *fh, int n, cudaStream_t s)
+                       void *fh, void *part, int n, cudaStream_t s)
 {
     if (n == 0) return LGF_OK;
+    if (const int grid = W2 ? 0 : gram_grid(ctx, n)) {
+        const int ph = prof_begin(ctx, s, "stage_force");
+        const lgf_status st = ctx->prec == LGF_F64 ? gram<double>(ctx, W1, U, ub, part, fh, n, grid, s)
+                                                   : gram<float>(ctx, W1, U, ub, part, fh, n, grid, s);
+        if (st != LGF_OK) return st;
+        LGF_CHECK_LAUNCH(ctx, "stage force solve");
+        prof_end(ctx, s, ph);
+        return LGF_OK;
+    }
     const unsigned gv = (unsigned)((n + 255) / 256), gn = (unsigned)((n + 7) / 8), gt = (unsigned)((n + 31) / 32);
     const int ph = prof_begin(ctx, s, "stage_force");
     if (ctx->prec == LGF_F64) {

@@ -89,3 +89,31 @@ def test_stage_empty_flow_set(ctx64):
     ctx64.nested_projection_stage(8, np.zeros((0, 3), np.int32), None, None, X_prev=X, X=X, ub=ub, W1=W, f=f)
     torch.cuda.synchronize()
     assert torch.equal(f, torch.zeros_like(f))
+
+
+@pytest.mark.parametrize("prec,nm,shift", [("f32", 1, 0), ("f32", 60, 0), ("f32", 60, 1), ("f32", 682, 0), ("f32", 683, 0),
+                                           ("f32", 1366, 0), ("f32", 2732, 0), ("f32", 5462, 0), ("f64", 1, 0),
+                                           ("f64", 341, 0), ("f64", 342, 1), ("f64", 1366, 0), ("f64", 2731, 0)])
+def test_stage_force_product_sizes(prec, nm, shift, ctx64, ctx32):
+    """f = W^T W (U - u_Gamma) with r = 0, so that U = 0 exactly: rows of every
+    length class of the one-pass product, rows that are no whole vectors, a
+    factor off the 16-byte alignment (shift) and rows beyond the one-pass limit.
+    Any summation order of n products meets 2 (n + 1) u |W|^T |W| |x| (u the
+    unit roundoff), with one more such factor for the second product."""
+    ctx = ctx64 if prec == "f64" else ctx32
+    dt, n = ctx.dtype, 3 * nm
+    b, D = 8, li.box_blocks(2, 2, 2)
+    gen = torch.Generator("cuda").manual_seed(nm)
+    X = 2.0 + 12.0 * torch.rand(nm, 3, dtype=torch.float64, device="cuda", generator=gen)
+    W = torch.randn(n * n + shift, dtype=dt, device="cuda", generator=gen)[shift:].view(n, n)
+    ub = torch.randn(n, dtype=dt, device="cuda", generator=gen)
+    r = torch.zeros(3 * D.shape[0] * b ** 3, dtype=dt, device="cuda")
+    u, f = torch.empty_like(r), torch.full((n,), float("nan"), dtype=dt, device="cuda")
+    ctx.nested_projection_stage(b, D, r, u, X_prev=X, X=X, ub=ub, W1=W, alpha=0.1, f=f)
+    ref, bound = torch.zeros(n, dtype=torch.float64, device="cuda"), torch.zeros(n, dtype=torch.float64, device="cuda")
+    for a in range(0, n, 2048):   # the rows in FP64, a part at a time
+        w = W[a:a + 2048].double()
+        ref -= w.T @ (w @ ub.double())
+        bound += w.abs().T @ (w.abs() @ ub.double().abs())
+    tol = 4 * (n + 2) * torch.finfo(dt).eps / 2
+    assert bool(((f.double() - ref).abs() <= tol * bound).all())
