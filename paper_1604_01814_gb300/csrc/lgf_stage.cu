@@ -128,9 +128,10 @@ __global__ void __launch_bounds__(256) k_gemv_t(const T *__restrict__ W, const T
     }
 }
 
-// f = W^T (W x), x = U - ub, in one pass over W (n x n, row-major), which the
-// two products read once each: HBM bounds both (15360^2 in FP32 is 944 MB, 139
-// us at the measured copy bandwidth).  A CTA of 512 threads holds a whole row
+// f = W^T (W x), x = U - ub, in one pass over W (n x n, row-major), which two
+// products read twice: HBM bounds both (15360^2 in FP32 is 944 MB, 139 us at
+// the measured copy bandwidth; two products took 450 us, one pass takes 172).
+// A CTA of 512 threads holds a whole row
 // in registers (NK 16-byte vectors per thread, the vectors of a warp
 // contiguous), forms y_r = W_r x, and adds y_r W_r to its own sum of W^T y, also in
 // registers; the next row is in flight meanwhile.  One barrier per row (the
