@@ -176,42 +176,6 @@ struct ColAddrW {   // element m of column w: m * W + w
     int W;
     __device__ __forceinline__ int operator()(int w, int m) const { return m * W + w; }
 };
-// Row-pass layout of element m of line l, chosen per length so that the
-// 8-byte accesses of every stage (first-stage stores at q G0 + g, middle
-// stage, last-stage groups at g RL + q, the Hermitian packing at the
-// digit-reversed positions) spread over the 16 bank pairs of a half-warp:
-// either padding, m + (m >> A) + (m >> B), or a swizzle of the low four
-// bits, m ^ (((m >> A) ^ (m >> B)) & 15) (a permutation inside each aligned
-// run of 16).  The (kind, A, B) per length came from a model of those
-// accesses that counts shared-memory wavefronts per half-warp; it cuts them
-// from 2.3x to 1.5x the conflict-free count on average.  B = 0: no second term.
-template <int ML>
-struct RowAddr {
-    static constexpr int KIND = ML == 512 || ML == 768 || ML == 1280 || ML == 1536 || ML == 2560 || ML == 3072 ||
-                                        ML == 4096
-                                    ? 1
-                                    : 0;   // 0 padding, 1 swizzle
-    static constexpr int A = ML == 32 || ML == 96 || ML == 160 || ML == 256 || ML == 512 || ML == 2048 || ML == 4096
-                                 ? 4
-                             : ML == 80 || ML == 1024 ? 3
-                             : ML == 768 || ML == 1536 || ML == 2560 || ML == 3072 ? 5
-                             : ML == 1280 ? 6
-                                          : 2;
-    static constexpr int B = ML == 80 || ML == 96 || ML == 512 || ML == 3072 ? 6
-                             : ML == 160 || ML == 1024 ? 7
-                             : ML == 2048 || ML == 4096 ? 8
-                                                        : 0;
-    // line stride: the largest index of a line plus one, plus one to offset lines
-    static constexpr int LD = (KIND == 0 ? ML + (ML >> A) + (B ? (ML >> B) : 0) : ML) + 1;
-    __device__ __forceinline__ int operator()(int l, int m) const
-    {
-        if constexpr (KIND == 0)
-            return l * LD + m + (m >> A) + (B ? (m >> B) : 0);
-        else
-            return l * LD + (m ^ (((m >> A) ^ (B ? (m >> B) : 0)) & 15));
-    }
-};
-
 template <typename T>
 __device__ __forceinline__ void load_twiddles(Cx<T> *tw, const Cx<T> *__restrict__ twg, int M)
 {
@@ -600,23 +564,152 @@ __global__ void __launch_bounds__(W * Plan<ML>::TPC, ConvOcc<T, ML, ZV>::value) 
 // ---------------------------------------------------------------------------
 // Row passes along x (real <-> half complex), two real rows per complex line.
 // ---------------------------------------------------------------------------
+// Layout and thread split of the x passes.  LPC lines (packed row pairs) share
+// a CTA and a line's M values are strided over shared memory: value r of
+// sub-problem q0 (position q0 N1 + r) of line l at base(q0) + r LD + l, LD odd.
+// Three access patterns have to be free of bank conflicts (16 lanes of 8 bytes):
+//   - the middle and last stages, lanes on consecutive lines, then on
+//     consecutive sub-problems: 16 lines are contiguous; with 8 or 4 lines,
+//     base() steps by LPC modulo 16 over the next 2 or 4 sub-problems;
+//   - the first stage, lanes on consecutive groups (so that the global accesses
+//     of the same thread are contiguous along x): stride LD, odd;
+//   - the pass over the half spectrum, lanes on consecutive frequencies k =
+//     q0 + R0 q1 + R0 R1 qL: base(q0) congruent to C1 (q0 mod 2^SH) +
+//     C2 (q0 >> SH) modulo 16, chosen per plan so that 16 consecutive k fall on
+//     16 different banks.
+// Every address is a thread constant plus a compile-time offset.
+// The passes are bound by shared-memory wavefronts and latency.  With every line
+// contiguous (padded or swizzled per length) and its threads side by side, 62 %
+// of the x inverse's wavefronts at length 640 were conflicts and it fetched
+// every half spectrum twice (for k and M - k): refresh of 556 blocks (length 640)
+// x inverse 101 -> 66 us, x forward 68 -> 53; 64-plate batch 797 -> 672 and 384 ->
+// 346 us; 512x256x256 wake (length 1024) x inverse 762 -> 656 us, x forward 634 -> 648.
+constexpr int congruent(int v, int c) { return v + (((c - v) % 16) + 16) % 16; }   // smallest >= v equal to c mod 16
+
+template <typename T, int ML>
+struct RowLay {
+    using P = Plan<ML>;
+    // threads per line: 16 to 24 values each (a masked last round where TPC
+    // does not divide the first stage's groups); TPC is a multiple of R0 in the
+    // three-stage plans
+    static constexpr int TPC = ML <= 32 || ML == 80 ? 4
+                             : ML <= 160 ? 8
+                             : ML <= 384 ? 16
+                             : ML <= 768 || ML == 1280 ? 32
+                             : ML == 2048 || ML == 4096 ? 128
+                                         : 64;
+    // lines per CTA: 16 up to length 768 while two CTAs fit an SM's shared
+    // memory (32 for the shortest lines, which would leave a CTA of two warps);
+    // 4 above, so that four CTAs of an SM overlap their loads, stages and
+    // stores (8 lines and two CTAs at length 1024: the x forward of the
+    // 512x256x256 wake took 804 us)
+    static constexpr int SIZE = int(sizeof(Cx<T>));
+    static constexpr bool fit(int l) { return (ML * (l + 1) + 64 + ML) * SIZE <= 112 * 1024; }
+    static constexpr int LPC = TPC == 4 ? 32
+                             : ML <= 768 && fit(16) ? 16
+                             : (ML <= 768 || ML == 1280) && fit(8) ? 8
+                             : fit(4) ? 4 : ML * SIZE <= 48 * 1024 ? 2 : 1;
+    static constexpr int LD = LPC > 1 ? LPC + 1 : 1;
+    static constexpr bool FEW = LPC < 16 && P::R0 >= 8;
+    static constexpr int C1 = FEW ? LPC : P::R0 == 16 ? 1
+                            : P::R0 == 8 ? (P::NST == 2 ? 2 : 1)
+                            : P::NST == 2 ? 4 : ML == 96 ? 2 : 1;
+    static constexpr int SH = FEW ? (LPC == 8 ? 1 : LPC == 4 ? 2 : 3) : P::R0 == 16 ? 4
+                            : P::R0 == 8 ? (P::NST == 2 || P::RL == 8 ? 3 : 2)
+                            : ML == 96 ? 1 : 2;
+    static constexpr int S1 = congruent(P::N1 * LD, C1);
+    static constexpr int S2 = congruent(((1 << SH) - 1) * S1 + P::N1 * LD, FEW ? 1 : 8);
+    static __host__ __device__ constexpr int base(int q0) { return (q0 & ((1 << SH) - 1)) * S1 + (q0 >> SH) * S2; }
+    static constexpr int THREADS = LPC * TPC;
+    static constexpr size_t SMEM = sizeof(Cx<T>) * (size_t)(ML + base(P::R0 - 1) + P::N1 * LD);
+    // resident CTAs the register allocation must allow: FP32 up to 1024 threads
+    // per SM (64 registers), FP64 leaves it to the compiler
+    static constexpr int BYSMEM = int(227 * 1024 / (SMEM + 1024)), BYREG = 1024 / THREADS;
+    static constexpr int OCC = sizeof(T) == 8 ? 1 : BYSMEM < BYREG ? (BYSMEM < 1 ? 1 : BYSMEM) : (BYREG < 1 ? 1 : BYREG);
+    static_assert(SMEM <= 227 * 1024 && THREADS <= 1024, "a CTA's lines fit");
+    static_assert(TPC % P::R0 == 0 || P::NST == 2, "the middle stage owns a sub-problem per thread");
+    // slot of frequency k
+    static __device__ __forceinline__ int freq_slot(int k)
+    {
+        const int q0 = k % P::R0, q1 = k / P::R0 % P::R1, qL = k / (P::R0 * P::R1);
+        return base(q0) + (q1 * P::RL + qL) * LD;
+    }
+};
+
+// The stages between the first one and the spectrum, lanes on consecutive
+// lines: DIR < 0 middle then last stage, DIR > 0 last then middle, all in
+// shared memory.  Barriers between and after the stages.
+template <typename T, int ML, int DIR>
+__device__ __forceinline__ void row_inner_stages(Cx<T> *__restrict__ s, const Cx<T> *__restrict__ tw)
+{
+    using P = Plan<ML>;
+    using L = RowLay<T, ML>;
+    constexpr int RL = P::RL, LD = L::LD;
+    const int l = threadIdx.x % L::LPC, t = threadIdx.x / L::LPC;
+    auto last = [&]() {
+#pragma unroll
+        for (int i = 0; i < (P::GL + L::TPC - 1) / L::TPC; ++i) {
+            const int g = t + i * L::TPC;
+            if (P::GL % L::TPC != 0 && g >= P::GL) break;
+            Cx<T> *p = s + L::base(g % P::R0) + (g / P::R0) * RL * LD + l;
+            Cx<T> c[RL];
+#pragma unroll
+            for (int q = 0; q < RL; ++q) c[q] = p[q * LD];
+            Dft<RL, DIR, T>::run(c);
+#pragma unroll
+            for (int q = 0; q < RL; ++q) p[q * LD] = c[q];
+        }
+        __syncthreads();
+    };
+    auto middle = [&]() {
+        if constexpr (P::NST == 3) {
+            constexpr int R = P::R1, NP = RL, TJ = L::TPC / P::R0;
+            static_assert(NP % TJ == 0, "whole groups per thread");
+            const int j0 = t / P::R0;
+            Cx<T> *p = s + L::base(t % P::R0) + j0 * LD + l;
+            const Cx<T> *tw1 = tw + P::TW1 + j0;
+#pragma unroll
+            for (int j = 0; j < NP; j += TJ) {
+                Cx<T> a[R];
+#pragma unroll
+                for (int q = 0; q < R; ++q) a[q] = p[(j + q * NP) * LD];
+                if (DIR < 0)
+                    dif_group<R, NP>(a, j, tw1);
+                else
+                    dit_group<R, NP>(a, j, tw1);
+#pragma unroll
+                for (int q = 0; q < R; ++q) p[(j + q * NP) * LD] = a[q];
+            }
+            __syncthreads();
+        }
+    };
+    if (DIR < 0) {
+        middle();
+        last();
+    } else {
+        last();
+        middle();
+    }
+}
+
 // Forward: rows (y, y+1) of source plane z, x in [s0x, s0x + Lsx), from the
 // block layout (HALF: the apply, where the row lies in [0, M/2) so the first
 // stage's upper inputs are zero at compile time) or from a dense box with row
 // length dense_ld (the spectrum build, full rows).
-template <typename T, int ML, int LPC, bool HALF>
+template <typename T, int ML, bool HALF>
 __device__ __forceinline__ void row_forward_body(int bx, int by, const T *__restrict__ f, Cx<T> *__restrict__ A,
                                                  const PoissonGeom &g, const Cx<T> *__restrict__ twg, int npairs,
                                                  int lb, int dense_ld)
 {
     using P = Plan<ML>;
-    constexpr int M = P::M;
+    using L = RowLay<T, ML>;
+    constexpr int M = P::M, TPC = L::TPC;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     Cx<T> *tw = reinterpret_cast<Cx<T> *>(smem_raw);
     Cx<T> *s = tw + M;
     load_twiddles(tw, twg, M);
-    const int t = threadIdx.x % P::TPC, l = threadIdx.x / P::TPC;
-    const int pr = bx * LPC + l;
+    const int t = threadIdx.x % TPC, l = threadIdx.x / TPC;
+    const int pr = bx * L::LPC + l;
     const bool live = pr < npairs;
     const int hp = g.Ls[1] >> 1;
     const int zi = live ? pr / hp : 0, yi = live ? 2 * (pr - zi * hp) : 0;
@@ -624,9 +717,9 @@ __device__ __forceinline__ void row_forward_body(int bx, int by, const T *__rest
     // nothing to transform (the y pass does not read those rows)
     if (g.srcrow && !__syncthreads_or(live && ((g.srcrow[zi >> lb] >> (yi >> lb)) & 1ull))) return;
     const T *ff = f + by * g.fstride;
-    const RowAddr<ML> ad{};
     constexpr int R0 = P::R0;
-    constexpr int NG0 = P::G0 / P::TPC;
+    constexpr int NG0 = (P::G0 + TPC - 1) / TPC;
+    constexpr bool MASKED = P::G0 % TPC != 0;   // the last round of groups is partial
     Cx<T> a[NG0][R0];
     if constexpr (HALF) {
         // the block-map row and the in-block offset of rows (y, y+1) are
@@ -636,12 +729,12 @@ __device__ __forceinline__ void row_forward_body(int bx, int by, const T *__rest
         const int inner = (((zi & bm) << lb) + (yi & bm)) << lb;
 #pragma unroll
         for (int i = 0; i < NG0; ++i) {
-            const int xr = t + i * P::TPC - g.s0[0];
+            const int xr = t + i * TPC - g.s0[0];
 #pragma unroll
             for (int p = 0; p < R0 / 2; ++p) {
                 const int x = xr + p * P::G0;
                 Cx<T> v{T(0), T(0)};
-                if (live && (unsigned)x < (unsigned)g.Ls[0]) {
+                if (live && (unsigned)x < (unsigned)g.Ls[0] && (!MASKED || t + i * TPC < P::G0)) {
                     const int bi = mrow[x >> lb];
                     if (bi >= 0) {
                         const T *q = ff + ((int64_t)bi << (3 * lb)) + inner + (x & bm);
@@ -655,13 +748,13 @@ __device__ __forceinline__ void row_forward_body(int bx, int by, const T *__rest
     } else {
 #pragma unroll
         for (int i = 0; i < NG0; ++i) {
-            const int gg = t + i * P::TPC;
+            const int gg = t + i * TPC;
             const T *row = ff + ((int64_t)(g.s0[2] + zi) * g.M[1] + (g.s0[1] + yi)) * dense_ld;
 #pragma unroll
             for (int p = 0; p < R0; ++p) {
                 const int x = gg + p * P::G0;
                 Cx<T> v{T(0), T(0)};
-                if (live && x >= g.s0[0] && x < g.s0[0] + g.Ls[0]) {
+                if (live && x >= g.s0[0] && x < g.s0[0] + g.Ls[0] && (!MASKED || gg < P::G0)) {
                     v.x = row[x];
                     v.y = row[dense_ld + x];
                 }
@@ -675,47 +768,39 @@ __device__ __forceinline__ void row_forward_body(int bx, int by, const T *__rest
     const bool single = HALF && g.s0[0] + g.Ls[0] <= P::G0;
 #pragma unroll
     for (int i = 0; i < NG0; ++i) {
-        const int gg = t + i * P::TPC;
+        const int gg = t + i * TPC;
+        if (MASKED && gg >= P::G0) break;
         if (single)
             dif_group_single<P::R0, P::G0>(a[i], gg, tw);
         else
             dif_group<P::R0, P::G0, HALF>(a[i], gg, tw);
 #pragma unroll
-        for (int q = 0; q < R0; ++q) s[ad(l, q * P::G0 + gg)] = a[i][q];
+        for (int q = 0; q < R0; ++q) s[L::base(q) + gg * L::LD + l] = a[i][q];
     }
     __syncthreads();
-    if constexpr (P::NST == 3) {
-        middle_stage<ML, -1>(s, ad, l, t, tw);
-        __syncthreads();
-    }
-    constexpr int RL = P::RL;
-#pragma unroll
-    for (int gg = t; gg < P::GL; gg += P::TPC) {
-        Cx<T> c[RL];
-#pragma unroll
-        for (int q = 0; q < RL; ++q) c[q] = s[ad(l, (gg * P::RL) + q)];
-        Dft<RL, -1, T>::run(c);
-#pragma unroll
-        for (int q = 0; q < RL; ++q) s[ad(l, (gg * P::RL) + q)] = c[q];
-    }
-    __syncthreads();
+    row_inner_stages<T, ML, -1>(s, tw);
     if (!live) return;
-    const int K = g.Kx;
+    // the two rows' half spectra from the packed line
+    constexpr int K = M / 2 + 1;
     Cx<T> *row = A + by * g.Astride + ((int64_t)zi * g.ldA_y + yi) * K;
-    for (int k = t; k < K; k += P::TPC) {
-        const Cx<T> zk = s[ad(l, pos_of<ML>(k))];
-        const Cx<T> zm = s[ad(l, pos_of<ML>(k == 0 ? 0 : M - k))];
+    const Cx<T> *sl = s + l;
+    auto unpack = [&](int k) {
+        const Cx<T> zk = sl[L::freq_slot(k)];
+        const Cx<T> zm = sl[L::freq_slot(k == 0 ? 0 : M - k)];
         row[k] = Cx<T>{T(0.5) * (zk.x + zm.x), T(0.5) * (zk.y - zm.y)};
         row[K + k] = Cx<T>{T(0.5) * (zk.y + zm.y), T(-0.5) * (zk.x - zm.x)};
-    }
+    };
+#pragma unroll 4
+    for (int i = 0; i < M / 2 / TPC; ++i) unpack(t + i * TPC);
+    if (t == 0) unpack(M / 2);
 }
 
-template <typename T, int ML, int LPC, bool HALF>
-__global__ void __launch_bounds__(LPC * Plan<ML>::TPC) k_row_forward(const T *__restrict__ f, Cx<T> *__restrict__ A,
-                                                                       PoissonGeom g, const Cx<T> *__restrict__ twg,
-                                                                       int npairs, int lb, int dense_ld)
+template <typename T, int ML, bool HALF>
+__global__ void __launch_bounds__(RowLay<T, ML>::THREADS, RowLay<T, ML>::OCC)
+    k_row_forward(const T *__restrict__ f, Cx<T> *__restrict__ A, PoissonGeom g, const Cx<T> *__restrict__ twg,
+                  int npairs, int lb, int dense_ld)
 {
-    row_forward_body<T, ML, LPC, HALF>(blockIdx.x, blockIdx.y, f, A, g, twg, npairs, lb, dense_ld);
+    row_forward_body<T, ML, HALF>(blockIdx.x, blockIdx.y, f, A, g, twg, npairs, lb, dense_ld);
 }
 
 // Inverse: rows (y, y+1) of target plane z from their half spectra; x in
@@ -723,100 +808,72 @@ __global__ void __launch_bounds__(LPC * Plan<ML>::TPC) k_row_forward(const T *__
 // HALF_OUT: the target x lies in [0, M/2) (even embedding), so only the
 // lower half of the last stage's outputs is formed; otherwise (the shifted x
 // window, targets up to M) every output is.
-// One line pair per slot l < LPC (thread t of TPC in it): rows (yi, yi+1)
-// of target plane zi, their half spectra at row[0..K) and row[K..2K), in any
-// memory; the Hermitian extension goes to s, the inverse sweep runs, and x in
-// [t0x, t0x + Ltx) scaled by dx^2 is scattered to the target blocks of uu.
-// tw holds the M twiddles in shared memory.  GUARD (the fused inverse, rows
-// in shared memory): the CTA may have threads beyond the LPC slots, which
-// take part in the barriers only.
-template <typename T, int ML, int LPC, bool HALF_OUT, bool GUARD = false>
-__device__ __forceinline__ void row_inverse_line(int t, int l, bool live, int zi, int yi,
-                                                 const Cx<T> *__restrict__ row, T *__restrict__ uu,
-                                                 const PoissonGeom &g, const Cx<T> *__restrict__ tw,
-                                                 Cx<T> *__restrict__ s, int lb)
+template <typename T, int ML, bool HALF_OUT>
+__device__ __forceinline__ void row_inverse_body(int bx, int by, const Cx<T> *__restrict__ A, T *__restrict__ u,
+                                                 const PoissonGeom &g, const Cx<T> *__restrict__ twg, int npairs,
+                                                 int lb)
 {
     using P = Plan<ML>;
-    constexpr int M = P::M;
-    const bool act = !GUARD || l < LPC;
-    if (GUARD) live = live && act;
-    const int K = g.Kx;
-    const RowAddr<ML> ad{};
-    // Hermitian extension of the two half spectra, packed as Z = G1 + i G2,
-    // stored at the digit-reversed positions the inverse sweep expects.
-    constexpr int NPT = M / P::TPC;
-    if constexpr (GUARD) {
-        // (row may lie in shared memory: each value is stored right after its
-        // load, so no long run of loads is held in registers)
-        if (act) {
+    using L = RowLay<T, ML>;
+    constexpr int M = P::M, TPC = L::TPC, K = M / 2 + 1;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    Cx<T> *tw = reinterpret_cast<Cx<T> *>(smem_raw);
+    Cx<T> *s = tw + M;
+    load_twiddles(tw, twg, M);
+    const int t = threadIdx.x % TPC, l = threadIdx.x / TPC;
+    const int pr = bx * L::LPC + l;
+    const bool live = pr < npairs;
+    const int hp = g.Lt[1] >> 1;
+    const int zi = live ? pr / hp : 0, yi = live ? 2 * (pr - zi * hp) : 0;
+    // a CTA whose lines all lie in row blocks without target blocks has
+    // nothing to write
+    if (g.tgtrow && !__syncthreads_or(live && ((g.tgtrow[zi >> lb] >> (yi >> lb)) & 1ull))) return;
+    // Hermitian extension of the two half spectra, packed as Z = G1 + i G2: the
+    // values at k give Z at k and at M - k, stored at the positions the inverse
+    // sweep expects; NB loads of each row in flight
+    const Cx<T> *row = A + by * g.Astride + ((int64_t)zi * g.ldA_y + yi) * K;
+    Cx<T> *sl = s + l;
+    constexpr int NI = M / 2 / TPC, NB = NI % 8 == 0 ? 8 : NI % 6 == 0 ? 6 : NI % 5 == 0 ? 5 : NI % 4 == 0 ? 4 : 1;
+    if (live) {
+        const Cx<T> e1 = t == 0 ? row[M / 2] : Cx<T>{T(0), T(0)};
+        const Cx<T> e2 = t == 0 ? row[K + M / 2] : Cx<T>{T(0), T(0)};
+#pragma unroll 1
+        for (int i0 = 0; i0 < NI; i0 += NB) {
+            Cx<T> g1[NB], g2[NB];
 #pragma unroll
-            for (int i = 0; i < NPT; ++i) {
-                const int k = t + i * P::TPC;
-                const int kk = k <= M / 2 ? k : M - k;
-                Cx<T> g1 = live ? row[kk] : Cx<T>{T(0), T(0)};
-                Cx<T> g2 = live ? row[K + kk] : Cx<T>{T(0), T(0)};
-                if (k == 0 || k == M / 2) {
-                    g1.y = T(0);
-                    g2.y = T(0);
-                }
-                s[ad(l, pos_of<ML>(k))] = k <= M / 2 ? Cx<T>{g1.x - g2.y, g1.y + g2.x} : Cx<T>{g1.x + g2.y, g2.x - g1.y};
+            for (int i = 0; i < NB; ++i) {
+                g1[i] = row[t + (i0 + i) * TPC];
+                g2[i] = row[K + t + (i0 + i) * TPC];
+            }
+#pragma unroll
+            for (int i = 0; i < NB; ++i) {
+                const int k = t + (i0 + i) * TPC;
+                if (k == 0) g1[i].y = g2[i].y = T(0);
+                sl[L::freq_slot(k)] = Cx<T>{g1[i].x - g2[i].y, g1[i].y + g2[i].x};
+                if (k != 0) sl[L::freq_slot(M - k)] = Cx<T>{g1[i].x + g2[i].y, g2[i].x - g1[i].y};
             }
         }
+        if (t == 0) sl[L::freq_slot(M / 2)] = Cx<T>{e1.x, e2.x};
     } else {
-        Cx<T> g1[NPT], g2[NPT];
-#pragma unroll
-        for (int i = 0; i < NPT; ++i) {
-            const int k = t + i * P::TPC;
-            const int kk = k <= M / 2 ? k : M - k;
-            g1[i] = live ? row[kk] : Cx<T>{T(0), T(0)};
-            g2[i] = live ? row[K + kk] : Cx<T>{T(0), T(0)};
-        }
-#pragma unroll
-        for (int i = 0; i < NPT; ++i) {
-            const int k = t + i * P::TPC;
-            Cx<T> v;
-            if (k <= M / 2) {
-                if (k == 0 || k == M / 2) {
-                    g1[i].y = T(0);
-                    g2[i].y = T(0);
-                }
-                v = {g1[i].x - g2[i].y, g1[i].y + g2[i].x};
-            } else {
-                v = {g1[i].x + g2[i].y, g2[i].x - g1[i].y};
-            }
-            s[ad(l, pos_of<ML>(k))] = v;
-        }
+        for (int k = t; k < M; k += TPC) sl[L::freq_slot(k)] = Cx<T>{T(0), T(0)};
     }
     __syncthreads();
-    constexpr int RL = P::RL;
-    if (act) {
-#pragma unroll
-        for (int gg = t; gg < P::GL; gg += P::TPC) {
-            Cx<T> c[RL];
-#pragma unroll
-            for (int q = 0; q < RL; ++q) c[q] = s[ad(l, (gg * P::RL) + q)];
-            Dft<RL, 1, T>::run(c);
-#pragma unroll
-            for (int q = 0; q < RL; ++q) s[ad(l, (gg * P::RL) + q)] = c[q];
-        }
-    }
-    __syncthreads();
-    if constexpr (P::NST == 3) {
-        if (act) middle_stage<ML, 1>(s, ad, l, t, tw);
-        __syncthreads();
-    }
+    row_inner_stages<T, ML, 1>(s, tw);
     if (!live) return;
     const T sc = T(g.scale);
     const int bm = g.b - 1;
     const int *mrow = g.tgtmap + ((zi >> lb) * g.nbt[1] + (yi >> lb)) * g.nbt[0];
     const int inner = (((zi & bm) << lb) + (yi & bm)) << lb;
+    T *uu = u + by * g.ustride;
     constexpr int R0 = P::R0;
     constexpr int NOUT = HALF_OUT ? R0 / 2 : R0;
 #pragma unroll
-    for (int gg = t; gg < P::G0; gg += P::TPC) {
+    for (int i = 0; i < (P::G0 + TPC - 1) / TPC; ++i) {
+        const int gg = t + i * TPC;
+        if (P::G0 % TPC != 0 && gg >= P::G0) break;
         Cx<T> a[R0];
 #pragma unroll
-        for (int q = 0; q < R0; ++q) a[q] = s[ad(l, q * P::G0 + gg)];
+        for (int q = 0; q < R0; ++q) a[q] = sl[L::base(q) + gg * L::LD];
         dit_group<P::R0, P::G0, HALF_OUT>(a, gg, tw);
         const int xr = gg - g.t0[0];
 #pragma unroll
@@ -832,35 +889,12 @@ __device__ __forceinline__ void row_inverse_line(int t, int l, bool live, int zi
     }
 }
 
-template <typename T, int ML, int LPC, bool HALF_OUT>
-__device__ __forceinline__ void row_inverse_body(int bx, int by, const Cx<T> *__restrict__ A, T *__restrict__ u,
-                                                 const PoissonGeom &g, const Cx<T> *__restrict__ twg, int npairs,
-                                                 int lb)
+template <typename T, int ML, bool HALF_OUT>
+__global__ void __launch_bounds__(RowLay<T, ML>::THREADS, RowLay<T, ML>::OCC)
+    k_row_inverse(const Cx<T> *__restrict__ A, T *__restrict__ u, PoissonGeom g, const Cx<T> *__restrict__ twg,
+                  int npairs, int lb)
 {
-    using P = Plan<ML>;
-    constexpr int M = P::M;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    Cx<T> *tw = reinterpret_cast<Cx<T> *>(smem_raw);
-    Cx<T> *s = tw + M;
-    load_twiddles(tw, twg, M);
-    const int t = threadIdx.x % P::TPC, l = threadIdx.x / P::TPC;
-    const int pr = bx * LPC + l;
-    const bool live = pr < npairs;
-    const int hp = g.Lt[1] >> 1;
-    const int zi = live ? pr / hp : 0, yi = live ? 2 * (pr - zi * hp) : 0;
-    // a CTA whose lines all lie in row blocks without target blocks has
-    // nothing to write
-    if (g.tgtrow && !__syncthreads_or(live && ((g.tgtrow[zi >> lb] >> (yi >> lb)) & 1ull))) return;
-    const Cx<T> *row = A + by * g.Astride + ((int64_t)zi * g.ldA_y + yi) * g.Kx;
-    row_inverse_line<T, ML, LPC, HALF_OUT>(t, l, live, zi, yi, row, u + by * g.ustride, g, tw, s, lb);
-}
-
-template <typename T, int ML, int LPC, bool HALF_OUT>
-__global__ void __launch_bounds__(LPC * Plan<ML>::TPC) k_row_inverse(const Cx<T> *__restrict__ A, T *__restrict__ u,
-                                                                       PoissonGeom g, const Cx<T> *__restrict__ twg,
-                                                                       int npairs, int lb)
-{
-    row_inverse_body<T, ML, LPC, HALF_OUT>(blockIdx.x, blockIdx.y, A, u, g, twg, npairs, lb);
+    row_inverse_body<T, ML, HALF_OUT>(blockIdx.x, blockIdx.y, A, u, g, twg, npairs, lb);
 }
 
 // ---------------------------------------------------------------------------
@@ -925,21 +959,21 @@ struct ConvJob {
     int cta0, gx;
 };
 
-template <typename T, int ML, int LPC, bool HALF>
-__global__ void __launch_bounds__(LPC * Plan<ML>::TPC) k_row_forward_rag(const __grid_constant__ RagTable<RowJob<T>> t)
+template <typename T, int ML, bool HALF>
+__global__ void __launch_bounds__(RowLay<T, ML>::THREADS, RowLay<T, ML>::OCC) k_row_forward_rag(const __grid_constant__ RagTable<RowJob<T>> t)
 {
     const RowJob<T> &J = rag_job(t);
     const int c = (int)blockIdx.x - J.cta0;
-    row_forward_body<T, ML, LPC, HALF>(c % J.gx, c / J.gx, (const T *)J.in, (Cx<T> *)J.out, J.g, J.tw, J.npairs, J.lb,
+    row_forward_body<T, ML, HALF>(c % J.gx, c / J.gx, (const T *)J.in, (Cx<T> *)J.out, J.g, J.tw, J.npairs, J.lb,
                                        0);
 }
 
-template <typename T, int ML, int LPC, bool HALF_OUT>
-__global__ void __launch_bounds__(LPC * Plan<ML>::TPC) k_row_inverse_rag(const __grid_constant__ RagTable<RowJob<T>> t)
+template <typename T, int ML, bool HALF_OUT>
+__global__ void __launch_bounds__(RowLay<T, ML>::THREADS, RowLay<T, ML>::OCC) k_row_inverse_rag(const __grid_constant__ RagTable<RowJob<T>> t)
 {
     const RowJob<T> &J = rag_job(t);
     const int c = (int)blockIdx.x - J.cta0;
-    row_inverse_body<T, ML, LPC, HALF_OUT>(c % J.gx, c / J.gx, (const Cx<T> *)J.in, (T *)J.out, J.g, J.tw, J.npairs,
+    row_inverse_body<T, ML, HALF_OUT>(c % J.gx, c / J.gx, (const Cx<T> *)J.in, (T *)J.out, J.g, J.tw, J.npairs,
                                            J.lb);
 }
 
@@ -980,16 +1014,6 @@ struct ColCfg {
     static constexpr int WMAX = int(98304 / (sizeof(Cx<T>) * ML)) < 1 ? 1 : int(98304 / (sizeof(Cx<T>) * ML));
     static constexpr int W = W0 < WMAX ? W0 : WMAX;
     static constexpr size_t SMEM = sizeof(Cx<T>) * (((size_t)ML) * (W + 1));
-};
-
-template <typename T, int ML>
-struct RowCfg {
-    static constexpr int TPC = Plan<ML>::TPC;
-    static constexpr int L0 = 256 / TPC < 1 ? 1 : (256 / TPC > 32 ? 32 : 256 / TPC);
-    static constexpr int LD = RowAddr<ML>::LD;
-    static constexpr int LMAX = int(98304 / (sizeof(Cx<T>) * LD)) < 1 ? 1 : int(98304 / (sizeof(Cx<T>) * LD));
-    static constexpr int LPC = L0 < LMAX ? L0 : LMAX;
-    static constexpr size_t SMEM = sizeof(Cx<T>) * (((size_t)ML) + (size_t)LPC * LD);
 };
 
 }  // namespace pk
@@ -1047,12 +1071,12 @@ template <typename T, int ML>
 lgf_status row_forward_m(lgf_ctx *ctx, const PoissonGeom &g, const T *f, Cx<T> *A, const Cx<T> *tw, int nfields,
                          int lb, int dense_ld, cudaStream_t s)
 {
-    using C = RowCfg<T, ML>;
-    auto kern = k_row_forward<T, ML, C::LPC, true>;
+    using C = RowLay<T, ML>;
+    auto kern = k_row_forward<T, ML, true>;
     if (dense_ld) {
         // full dense rows: only the FP64 spectrum build
         if constexpr (sizeof(T) == 8)
-            kern = k_row_forward<T, ML, C::LPC, false>;
+            kern = k_row_forward<T, ML, false>;
         else
             return fail(ctx, LGF_EINVAL, "row forward: FP32 dense rows");
     } else if (g.s0[0] < 0 || 2 * (g.s0[0] + g.Ls[0]) > g.M[0]) {
@@ -1063,7 +1087,7 @@ lgf_status row_forward_m(lgf_ctx *ctx, const PoissonGeom &g, const T *f, Cx<T> *
     const int npairs = (g.Ls[1] / 2) * g.Ls[2];
     dim3 grid((npairs + C::LPC - 1) / C::LPC, nfields);
     const int ph = prof_begin(ctx, s, dense_ld ? "spectrum_x_forward" : "poisson_x_forward");
-    kern<<<grid, C::LPC * C::TPC, C::SMEM, s>>>(f, A, g, tw, npairs, lb, dense_ld);
+    kern<<<grid, C::THREADS, C::SMEM, s>>>(f, A, g, tw, npairs, lb, dense_ld);
     LGF_CHECK_LAUNCH(ctx, "poisson x-forward");
     prof_end(ctx, s, ph);
     return LGF_OK;
@@ -1073,17 +1097,17 @@ template <typename T, int ML>
 lgf_status row_inverse_m(lgf_ctx *ctx, const PoissonGeom &g, const Cx<T> *A, T *u, const Cx<T> *tw, int nfields,
                          int lb, cudaStream_t s)
 {
-    using C = RowCfg<T, ML>;
-    auto kern = k_row_inverse<T, ML, C::LPC, true>;
+    using C = RowLay<T, ML>;
+    auto kern = k_row_inverse<T, ML, true>;
     if (g.t0[0] < 0 || g.t0[0] + g.Lt[0] > g.M[0])
         return fail(ctx, LGF_EINVAL, "row inverse: target beyond the transform length");
-    if (2 * (g.t0[0] + g.Lt[0]) > g.M[0]) kern = k_row_inverse<T, ML, C::LPC, false>;
+    if (2 * (g.t0[0] + g.Lt[0]) > g.M[0]) kern = k_row_inverse<T, ML, false>;
     lgf_status st = set_smem(ctx, kern, C::SMEM);
     if (st != LGF_OK) return st;
     const int npairs = (g.Lt[1] / 2) * g.Lt[2];
     dim3 grid((npairs + C::LPC - 1) / C::LPC, nfields);
     const int ph = prof_begin(ctx, s, "poisson_x_inverse");
-    kern<<<grid, C::LPC * C::TPC, C::SMEM, s>>>(A, u, g, tw, npairs, lb);
+    kern<<<grid, C::THREADS, C::SMEM, s>>>(A, u, g, tw, npairs, lb);
     LGF_CHECK_LAUNCH(ctx, "poisson x-inverse");
     prof_end(ctx, s, ph);
     return LGF_OK;
@@ -1187,8 +1211,8 @@ lgf_status rag_send(lgf_ctx *ctx, Kern kern, int threads, size_t smem, J *jobs, 
 template <typename T, int ML>
 lgf_status row_forward_rag_m(lgf_ctx *ctx, RowJob<T> *jobs, int n, cudaStream_t s)
 {
-    using C = RowCfg<T, ML>;
-    auto kern = k_row_forward_rag<T, ML, C::LPC, true>;
+    using C = RowLay<T, ML>;
+    auto kern = k_row_forward_rag<T, ML, true>;
     for (int i = 0; i < n; ++i) {
         const PoissonGeom &g = jobs[i].g;
         if (g.M[0] != ML || g.s0[0] < 0 || 2 * (g.s0[0] + g.Ls[0]) > g.M[0])
@@ -1197,14 +1221,14 @@ lgf_status row_forward_rag_m(lgf_ctx *ctx, RowJob<T> *jobs, int n, cudaStream_t 
     }
     lgf_status st = set_smem(ctx, kern, C::SMEM);
     if (st != LGF_OK) return st;
-    return rag_send(ctx, kern, C::LPC * C::TPC, C::SMEM, jobs, n, s, "poisson_x_forward");
+    return rag_send(ctx, kern, C::THREADS, C::SMEM, jobs, n, s, "poisson_x_forward");
 }
 
 template <typename T, int ML>
 lgf_status row_inverse_rag_m(lgf_ctx *ctx, bool half_out, RowJob<T> *jobs, int n, cudaStream_t s)
 {
-    using C = RowCfg<T, ML>;
-    auto kern = half_out ? k_row_inverse_rag<T, ML, C::LPC, true> : k_row_inverse_rag<T, ML, C::LPC, false>;
+    using C = RowLay<T, ML>;
+    auto kern = half_out ? k_row_inverse_rag<T, ML, true> : k_row_inverse_rag<T, ML, false>;
     for (int i = 0; i < n; ++i) {
         const PoissonGeom &g = jobs[i].g;
         if (g.M[0] != ML || g.t0[0] < 0 || g.t0[0] + g.Lt[0] > g.M[0] ||
@@ -1214,7 +1238,7 @@ lgf_status row_inverse_rag_m(lgf_ctx *ctx, bool half_out, RowJob<T> *jobs, int n
     }
     lgf_status st = set_smem(ctx, kern, C::SMEM);
     if (st != LGF_OK) return st;
-    return rag_send(ctx, kern, C::LPC * C::TPC, C::SMEM, jobs, n, s, "poisson_x_inverse");
+    return rag_send(ctx, kern, C::THREADS, C::SMEM, jobs, n, s, "poisson_x_inverse");
 }
 
 template <typename T, int ML>
