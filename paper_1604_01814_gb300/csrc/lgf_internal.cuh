@@ -22,6 +22,7 @@ constexpr int kMinTableRadius = 24;  // expansion error at |n| > 24 is below 1e-
 // Transform lengths: 2^k, 3 * 2^k and 5 * 2^k from 32 to 4096.
 // --------------------------------------------------------------------------
 int next_fft_size(int n);   // smallest supported length >= n
+int row_stride(int K);      // storage for a row of K values (see there)
 // --------------------------------------------------------------------------
 // Poisson plan: one problem's padded transform box.
 // Box coordinates are lattice coordinates minus `lo` (the union bounding box
@@ -30,6 +31,7 @@ int next_fft_size(int n);   // smallest supported length >= n
 struct PoissonGeom {
     int M[3];           // transform lengths (x, y, z)
     int Kx;             // Mx / 2 + 1 (half spectrum along x)
+    int ld;             // row stride of A, B and the kernel spectrum (row_stride(Kx))
     int s0[3], Ls[3];   // source region [s0, s0 + Ls) in box coordinates
     int t0[3], Lt[3];   // target region
     int b;

@@ -229,11 +229,11 @@ __global__ void __cluster_dims__(NCL, 1, 1) __launch_bounds__(YXCfg<MY, MX>::THR
         const ColAddrW ad{W};
         const int w = threadIdx.x % W, t = threadIdx.x / W;
         const bool act = !GY || t < PY::TPC;
-        const Cx<T> *plane = J.B + field * g.Bstride + (int64_t)zi * MY * K;
+        const Cx<T> *plane = J.B + field * g.Bstride + (int64_t)zi * MY * g.ld;
         const bool half = lo + n <= MY / 2;
         constexpr int RL = PY::RL, R0 = PY::R0;
         constexpr int NGL = PY::GL / PY::TPC;
-        const int64_t istep = (int64_t)(MY / RL) * K;
+        const int64_t istep = (int64_t)(MY / RL) * g.ld;
         const int ntile = (K + W - 1) / W;
 #pragma unroll 1
         for (int tile = rank; tile < ntile; tile += NCL) {
@@ -244,7 +244,7 @@ __global__ void __cluster_dims__(NCL, 1, 1) __launch_bounds__(YXCfg<MY, MX>::THR
 #pragma unroll
             for (int i = 0; i < NGL; ++i) {
                 const int gg = t + i * PY::TPC;
-                int64_t off = (int64_t)freq_of<MY>(gg * RL) * K;
+                int64_t off = (int64_t)freq_of<MY>(gg * RL) * g.ld;
 #pragma unroll
                 for (int q = 0; q < RL; ++q) {
                     cc[i][q] = live ? ldg_cx(ib + off) : Cx<T>{T(0), T(0)};

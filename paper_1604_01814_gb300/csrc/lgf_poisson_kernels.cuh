@@ -442,8 +442,8 @@ struct ConvOcc {
 // spectrum of the shifted y window ([kz][ky < My][kx], no mirror in ky).
 template <typename T, int ML, int W, int SPEC>
 __device__ __forceinline__ void col_convolve_body(int bx, int nf, Cx<T> *__restrict__ B, const void *__restrict__ specv,
-                                                  int K, int My, int s0, int ns, int t0, int nt, int64_t field,
-                                                  const Cx<T> *__restrict__ twg)
+                                                  int K, int ld, int lds, int My, int s0, int ns, int t0, int nt,
+                                                  int64_t field, const Cx<T> *__restrict__ twg)
 {
     constexpr bool CPLX = SPEC > 0;
     using SpecT = typename std::conditional<CPLX, Cx<T>, T>::type;
@@ -458,8 +458,8 @@ __device__ __forceinline__ void col_convolve_body(int bx, int nf, Cx<T> *__restr
     int kx, ky;
     const int field_i = bx % nf;
     const bool live = column_of<W>(bx / nf, w, K, My, kx, ky);
-    const int64_t plane = (int64_t)My * K;
-    Cx<T> *bb = B + field_i * field + (int64_t)ky * K + kx;
+    const int64_t plane = (int64_t)My * ld;
+    Cx<T> *bb = B + field_i * field + (int64_t)ky * ld + kx;
     const ColAddrW ad{W};
     constexpr int R0 = P::R0;
     constexpr int NG0 = P::G0 / P::TPC;
@@ -495,8 +495,8 @@ __device__ __forceinline__ void col_convolve_body(int bx, int nf, Cx<T> *__restr
     constexpr int S = M / RL;   // frequency step of the last stage's digit
     const int Khy = SPEC == 2 ? My : My / 2 + 1;
     const int kyr = SPEC == 2 ? ky : (ky <= My - ky ? ky : My - ky);
-    const SpecT *sp = spec + (int64_t)kyr * K + kx;
-    const int64_t sp_plane = (int64_t)Khy * K, sp_step = S * sp_plane;
+    const SpecT *sp = spec + (int64_t)kyr * lds + kx;
+    const int64_t sp_plane = (int64_t)Khy * lds, sp_step = S * sp_plane;
 #pragma unroll
     for (int g = t; g < P::GL; g += P::TPC) {
         // frequency of digit q: kb + q S; its mirror M - kb - q S once past M/2
@@ -554,11 +554,12 @@ __device__ __forceinline__ void col_convolve_body(int bx, int nf, Cx<T> *__restr
 
 template <typename T, int ML, int W, int SPEC, int ZV>
 __global__ void __launch_bounds__(W * Plan<ML>::TPC, ConvOcc<T, ML, ZV>::value) k_col_convolve(Cx<T> *__restrict__ B, const void *__restrict__ specv,
-                                                                      int K, int My, int s0, int ns, int t0, int nt,
-                                                                      int64_t field, const Cx<T> *__restrict__ twg)
+                                                                      int K, int ld, int lds, int My, int s0, int ns,
+                                                                      int t0, int nt, int64_t field,
+                                                                      const Cx<T> *__restrict__ twg)
 {
-    col_convolve_body<T, ML, W, SPEC>(blockIdx.x, gridDim.x / col_ctas<W>(K, My), B, specv, K, My, s0, ns, t0, nt,
-                                      field, twg);
+    col_convolve_body<T, ML, W, SPEC>(blockIdx.x, gridDim.x / col_ctas<W>(K, My), B, specv, K, ld, lds, My, s0, ns, t0,
+                                      nt, field, twg);
 }
 
 // ---------------------------------------------------------------------------
@@ -781,14 +782,13 @@ __device__ __forceinline__ void row_forward_body(int bx, int by, const T *__rest
     row_inner_stages<T, ML, -1>(s, tw);
     if (!live) return;
     // the two rows' half spectra from the packed line
-    constexpr int K = M / 2 + 1;
-    Cx<T> *row = A + by * g.Astride + ((int64_t)zi * g.ldA_y + yi) * K;
+    Cx<T> *row = A + by * g.Astride + ((int64_t)zi * g.ldA_y + yi) * g.ld, *row2 = row + g.ld;
     const Cx<T> *sl = s + l;
     auto unpack = [&](int k) {
         const Cx<T> zk = sl[L::freq_slot(k)];
         const Cx<T> zm = sl[L::freq_slot(k == 0 ? 0 : M - k)];
         row[k] = Cx<T>{T(0.5) * (zk.x + zm.x), T(0.5) * (zk.y - zm.y)};
-        row[K + k] = Cx<T>{T(0.5) * (zk.y + zm.y), T(-0.5) * (zk.x - zm.x)};
+        row2[k] = Cx<T>{T(0.5) * (zk.y + zm.y), T(-0.5) * (zk.x - zm.x)};
     };
 #pragma unroll 4
     for (int i = 0; i < M / 2 / TPC; ++i) unpack(t + i * TPC);
@@ -815,7 +815,7 @@ __device__ __forceinline__ void row_inverse_body(int bx, int by, const Cx<T> *__
 {
     using P = Plan<ML>;
     using L = RowLay<T, ML>;
-    constexpr int M = P::M, TPC = L::TPC, K = M / 2 + 1;
+    constexpr int M = P::M, TPC = L::TPC;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     Cx<T> *tw = reinterpret_cast<Cx<T> *>(smem_raw);
     Cx<T> *s = tw + M;
@@ -831,19 +831,19 @@ __device__ __forceinline__ void row_inverse_body(int bx, int by, const Cx<T> *__
     // Hermitian extension of the two half spectra, packed as Z = G1 + i G2: the
     // values at k give Z at k and at M - k, stored at the positions the inverse
     // sweep expects; NB loads of each row in flight
-    const Cx<T> *row = A + by * g.Astride + ((int64_t)zi * g.ldA_y + yi) * K;
+    const Cx<T> *row = A + by * g.Astride + ((int64_t)zi * g.ldA_y + yi) * g.ld, *row2 = row + g.ld;
     Cx<T> *sl = s + l;
     constexpr int NI = M / 2 / TPC, NB = NI % 8 == 0 ? 8 : NI % 6 == 0 ? 6 : NI % 5 == 0 ? 5 : NI % 4 == 0 ? 4 : 1;
     if (live) {
         const Cx<T> e1 = t == 0 ? row[M / 2] : Cx<T>{T(0), T(0)};
-        const Cx<T> e2 = t == 0 ? row[K + M / 2] : Cx<T>{T(0), T(0)};
+        const Cx<T> e2 = t == 0 ? row2[M / 2] : Cx<T>{T(0), T(0)};
 #pragma unroll 1
         for (int i0 = 0; i0 < NI; i0 += NB) {
             Cx<T> g1[NB], g2[NB];
 #pragma unroll
             for (int i = 0; i < NB; ++i) {
                 g1[i] = row[t + (i0 + i) * TPC];
-                g2[i] = row[K + t + (i0 + i) * TPC];
+                g2[i] = row2[t + (i0 + i) * TPC];
             }
 #pragma unroll
             for (int i = 0; i < NB; ++i) {
@@ -955,7 +955,7 @@ struct ConvJob {
     const void *spec;
     const Cx<T> *tw;
     int64_t field;
-    int K, My, s0, ns, t0, nt, nf;
+    int K, ld, lds, My, s0, ns, t0, nt, nf;
     int cta0, gx;
 };
 
@@ -1000,8 +1000,8 @@ __global__ void __launch_bounds__(W * Plan<ML>::TPC, ConvOcc<T, ML, ZV>::value) 
     const __grid_constant__ RagTable<ConvJob<T>> t)
 {
     const ConvJob<T> &J = rag_job(t);
-    col_convolve_body<T, ML, W, SPEC>((int)blockIdx.x - J.cta0, J.nf, J.B, J.spec, J.K, J.My, J.s0, J.ns, J.t0, J.nt,
-                                      J.field, J.tw);
+    col_convolve_body<T, ML, W, SPEC>((int)blockIdx.x - J.cta0, J.nf, J.B, J.spec, J.K, J.ld, J.lds, J.My, J.s0, J.ns,
+                                      J.t0, J.nt, J.field, J.tw);
 }
 
 // ---------------------------------------------------------------------------
@@ -1172,8 +1172,8 @@ lgf_status col_convolve_m(lgf_ctx *ctx, const PoissonGeom &g, Cx<T> *B, const T 
     if (st != LGF_OK) return st;
     dim3 grid(nfields * col_ctas<C::W>(g.Kx, g.M[1]));
     const int ph = prof_begin(ctx, s, "poisson_z_convolve");
-    kern<<<grid, C::W * C::TPC, C::SMEM, s>>>(B, spec, g.Kx, g.M[1], g.s0[2], g.Ls[2], g.t0[2], g.Lt[2], g.Bstride,
-                                              tw);
+    kern<<<grid, C::W * C::TPC, C::SMEM, s>>>(B, spec, g.Kx, g.ld, g.ld, g.M[1], g.s0[2], g.Ls[2], g.t0[2], g.Lt[2],
+                                              g.Bstride, tw);
     LGF_CHECK_LAUNCH(ctx, "poisson z-convolve");
     prof_end(ctx, s, ph);
     return LGF_OK;
