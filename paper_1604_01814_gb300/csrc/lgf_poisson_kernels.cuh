@@ -599,15 +599,16 @@ struct RowLay {
                              : ML <= 768 || ML == 1280 ? 32
                              : ML == 2048 || ML == 4096 ? 128
                                          : 64;
-    // lines per CTA: 16 up to length 768 while two CTAs fit an SM's shared
-    // memory (32 for the shortest lines, which would leave a CTA of two warps);
-    // 4 above, so that four CTAs of an SM overlap their loads, stages and
-    // stores (8 lines and two CTAs at length 1024: the x forward of the
-    // 512x256x256 wake took 804 us)
+    // lines per CTA: 8 up to length 768 (16 for the plans that start with radix 4,
+    // whose 8-line layout would meet conflicts; 32 for the shortest lines, which would
+    // leave a CTA of two warps), 4 above, so that several CTAs of an SM
+    // overlap their loads, stages and stores and a small box still fills the GPU: 16
+    // lines at length 256 took the 128^3 box's batch from 99.7 to 105.3 us, 8 lines
+    // at length 1024 the wake's x forward from 648 to 804 us
     static constexpr int SIZE = int(sizeof(Cx<T>));
     static constexpr bool fit(int l) { return (ML * (l + 1) + 64 + ML) * SIZE <= 112 * 1024; }
     static constexpr int LPC = TPC == 4 ? 32
-                             : ML <= 768 && fit(16) ? 16
+                             : ML <= 768 && P::R0 < 8 && fit(16) ? 16
                              : (ML <= 768 || ML == 1280) && fit(8) ? 8
                              : fit(4) ? 4 : ML * SIZE <= 48 * 1024 ? 2 : 1;
     static constexpr int LD = LPC > 1 ? LPC + 1 : 1;
