@@ -46,6 +46,19 @@ __device__ __forceinline__ void bulk_copy(void *dst_smem, const void *src_gmem, 
                  : "memory");
 }
 
+// Per-thread asynchronous copy of 16 bytes (both addresses 16-byte aligned),
+// or 16 zero bytes when !ok (src is then not read but must be a valid address).
+__device__ __forceinline__ void copy16(void *dst_smem, const void *src_gmem, bool ok)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_u32(dst_smem)), "l"(src_gmem),
+                 "r"(ok ? 16 : 0)
+                 : "memory");
+}
+
+// The calling thread's copy16 copies have landed (a barrier makes them
+// visible to the CTA).
+__device__ __forceinline__ void copies_done() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
 __device__ __forceinline__ bool mbar_try(uint64_t *bar, uint32_t parity)
 {
     uint32_t ok;

@@ -325,6 +325,90 @@ __global__ void __launch_bounds__(Cfg<T, LB, AX>::THREADS)
     }
 }
 
+// One 8-byte column element: two adjacent x values in FP32 (packed FMA), one in FP64.
+template <typename T>
+struct Col8;
+template <>
+struct Col8<float> {
+    using V = float2;
+    static constexpr int N = 2;
+    static __device__ __forceinline__ V fma(V w, V x, V a) { return __ffma2_rn(w, x, a); }
+};
+template <>
+struct Col8<double> {
+    using V = double;
+    static constexpr int N = 1;
+    static __device__ __forceinline__ V fma(V w, V x, V a) { return ::fma(w, x, a); }
+};
+
+// The z pass for block edges 16 and 32: a thread owns one 8-byte column of a
+// block and 16 outputs along z.  In the block layout a z-plane is contiguous, so the
+// loads of a warp are too, straight from global memory: the 16 + 2 RMAX planes
+// of the window come in chunks of 8, the next chunk in flight while the current one
+// feeds the 16 accumulators; no shared memory, no barrier.  Every input is
+// fetched (16 + 2 RMAX) / 16 times, from L2 or L1.  Staging slabs in shared memory with 4
+// outputs per thread read it (4 + 2 RMAX) / 4 times from there: the l1tex pipe was
+// 70 % busy and 556 blocks of 16^3 (3 fields, RMAX 8) took 16.2 us, now 12.3; the
+// 64-plate batch's launch 281, now 215.  Blocks of 8 keep the staged pass: a plane has
+// too few columns for a CTA.
+// The order of the additions is that of k_sep_win.
+template <typename T, int LB>
+struct ZCfg {
+    static constexpr int b = 1 << LB, V = 16;
+    static constexpr int LANES = b * b / Col8<T>::N;   // columns of a block
+    static constexpr int THREADS = LANES < 128 ? LANES : 128;
+    static constexpr int NY = (LANES / THREADS) * (b / V);   // grid.y: slices of the plane, runs along z
+};
+template <typename T, int LB, int RMAX, class Tab = SepJobs<T>>
+__global__ void __launch_bounds__(ZCfg<T, LB>::THREADS)
+    k_sep_z(const __grid_constant__ Tab jobs, const int *__restrict__ nbr_arg, int nr_arg)
+{
+    using C = ZCfg<T, LB>;
+    using CV = Col8<T>;
+    using VT = typename CV::V;
+    constexpr int b = C::b, bm = b - 1, V = C::V, NPOS = V + 2 * RMAX, CH = 8;
+    static_assert(NPOS % CH == 0, "whole chunks");
+    const SepAt<T> at = sep_at(jobs, nbr_arg, nullptr, nr_arg);
+    const SepJob<T> &J = *at.J;
+    const int slice = blockIdx.y % (C::LANES / C::THREADS);
+    const int z0 = blockIdx.y / (C::LANES / C::THREADS) * V;
+    const int off = (slice * C::THREADS + threadIdx.x) * CV::N;
+    const T *inf = J.in + at.field * J.in_stride + off;
+    const int *nb = at.nbr + (int64_t)at.item * (2 * at.nr + 1) + at.nr;
+    auto load = [&](VT (&v)[CH], int c) {
+#pragma unroll
+        for (int i = 0; i < CH; ++i) {
+            const int e = z0 + c * CH + i - RMAX;
+            const int bi = nb[e >> LB];
+            v[i] = bi >= 0 ? __ldg(reinterpret_cast<const VT *>(inf + ((int64_t)bi << (3 * LB)) + ((e & bm) << (2 * LB))))
+                           : VT{};
+        }
+    };
+    VT cur[CH], nxt[CH], acc[V];
+    load(cur, 0);
+    WinW<T, RMAX> W;
+    load_weights(W, J.w, J.R);
+#pragma unroll
+    for (int v = 0; v < V; ++v) acc[v] = VT{};
+#pragma unroll
+    for (int c = 0; c < NPOS / CH; ++c) {
+        if (c + 1 < NPOS / CH) load(nxt, c + 1);
+#pragma unroll
+        for (int i = 0; i < CH; ++i) {
+#pragma unroll
+            for (int v = 0; v < V; ++v) {
+                const int d = c * CH + i - RMAX - v;
+                if (d >= -RMAX && d <= RMAX) acc[v] = CV::fma(W.w[d < 0 ? -d : d], cur[i], acc[v]);
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < CH; ++i) cur[i] = nxt[i];
+    }
+    T *outf = J.out + at.field * J.out_stride + ((int64_t)at.item << (3 * LB)) + ((int64_t)z0 << (2 * LB)) + off;
+#pragma unroll
+    for (int v = 0; v < V; ++v) *reinterpret_cast<VT *>(outf + (v << (2 * LB))) = acc[v];
+}
+
 // The z pass as a persistent kernel that stages with bulk asynchronous
 // copies.  In the block layout every staged z-plane of a slab (NS rows of b)
 // is one contiguous run, so a slab plus its halo is at most E bulk copies
@@ -425,200 +509,150 @@ __global__ void __launch_bounds__(Cfg<T, LB, 2>::THREADS)
 
 // Fused x and y passes.  A CTA owns one output block, or two that are
 // neighbours in y (a pair shares the y halo between them: 2b + 2 RMAX staged
-// rows for 2b outputs instead of 2 (b + 2 RMAX)), and NS z-planes.  It stages
-// the neighbourhood from the xy neighbour blocks, runs the x stencil over
-// every staged row into an intermediate [NS][EY][b] and then the y stencil to
-// the output block(s).
+// rows for 2b outputs instead of 2 (b + 2 RMAX)), and NS z-planes.
+//   - The neighbourhood (rows of b + 2 RMAX values) comes by 16-byte
+//     asynchronous copies, zero-filled where a block is absent.
+//   - x stencil: a thread takes a row (half a row of 32), its window in
+//     registers, and writes the outputs over the start of the same row.
+//   - y stencil: a thread takes an 8-byte column and VY outputs along it.
+// Row pitch b + 2 RMAX plus 16 bytes: the 16-byte accesses of eight rows fall on
+// different banks; planes are skewed so that a half-warp's 8-byte columns do too.
+// Shared memory is what bounds it (88 % of l1tex before, when a thread made 4
+// outputs of each stencil): a window of 16 + 2 RMAX values feeds 16 outputs along
+// x and one of VY + 2 RMAX feeds VY along y, where (4 + 2 RMAX) / 4 values were
+// read per output.
+// 556 blocks of 16^3 (3 fields, RMAX 8): 38 -> 30 us; the 64-plate batch's launch
+// 712 -> 488 us.
 template <typename T, int LB, int RMAX>
 struct XYCfg {
     static constexpr int b = 1 << LB, E = b + 2 * RMAX;
     static constexpr int EY1 = b + 2 * RMAX, EY = 2 * b + 2 * RMAX;   // staged rows: single, pair
-    // FP32 stages row pairs interleaved, [EY/2][P2], with a 16-byte skew per
-    // row pair (pitch P2 = 2E + 4), so that the row pairs of a warp start on
-    // different bank groups.
-    static constexpr int P2 = 2 * E + 4;
-    static constexpr int RG = sizeof(T) == 4 ? (EY / 2) * P2 : EY * E;   // staged elements per plane
-    // pitch of the x stencil's output rows: 20 floats for FP32 16^3 blocks, so
-    // that the y stencil's two thread quads (rows 4 apart) fall on the two
-    // halves of the banks; b elsewhere
-    static constexpr int IP = sizeof(T) == 4 && b == 16 ? 20 : b;
-    static constexpr int per_plane = RG + EY * IP;
-    static constexpr int NS0 = 12288 / per_plane;
-    static constexpr int NS = NS0 >= 8 ? 8 : NS0 >= 4 ? 4 : NS0 >= 2 ? 2 : 1;
-    static constexpr int NSB = NS > b ? b : NS;
-    static constexpr size_t SMEM = sizeof(T) * (size_t)NSB * per_plane;
+    static constexpr int NV = 16 / (int)sizeof(T);
+    static constexpr int LD = E + NV;                                // row pitch
+    static constexpr int V = b < 16 ? b : 16, GX = b / V;            // x outputs per thread, threads per row
+    static constexpr int VY = 8, GY = b / VY;                        // y outputs per thread
+    static constexpr int NS = 8 * EY * GX <= 256 ? 8 : 4 * EY * GX <= 256 ? 4 : 2 * EY * GX <= 256 ? 2 : 1;
+    static constexpr int THREADS = (NS * EY * GX + 31) / 32 * 32;
+    static constexpr int RB = b * (int)sizeof(T);                    // bytes of a row of outputs
+    static constexpr int SKEW = RB >= 128 ? 0 : (RB + 128 - EY * LD * (int)sizeof(T) % 128) % 128 / (int)sizeof(T);
+    static constexpr int PL = EY * LD + SKEW;                        // plane pitch
+    static constexpr size_t SMEM = sizeof(T) * (size_t)NS * PL;
+    static_assert(THREADS <= 256 && b % NS == 0 && SKEW % NV == 0, "one row item per thread, aligned planes");
 };
+constexpr int kMaxWinNr = 2;   // neighbour blocks on a side: RMAX <= 16, b >= 8
 
 // items: [n][2] output blocks (second -1 for a single block); nbr: for every
 // output block its (2nr+1)^2 xy neighbourhood of source blocks.
 template <typename T, int LB, int RMAX, class Tab = SepJobs<T>>
-__global__ void __launch_bounds__(256) k_sep_xy(const __grid_constant__ Tab jobs, const int *__restrict__ nbr_arg,
-                                                const int *__restrict__ items_arg, int nr_arg)
+__global__ void __launch_bounds__(XYCfg<T, LB, RMAX>::THREADS)
+    k_sep_xy(const __grid_constant__ Tab jobs, const int *__restrict__ nbr_arg, const int *__restrict__ items_arg,
+             int nr_arg)
 {
     const SepAt<T> at = sep_at(jobs, nbr_arg, items_arg, nr_arg);
     const SepJob<T> &J = *at.J;
-    const int field = at.field;
-    const int *__restrict__ nbr = at.nbr;
-    const int *__restrict__ items = at.items;
     const int nr = at.nr;
-    const T *__restrict__ wg = J.w;
-    const int R = J.R;
     using C = XYCfg<T, LB, RMAX>;
     using VT = typename Vec<T>::V;
-    constexpr int b = C::b, bm = b - 1, NV = Vec<T>::N, NS = C::NSB, HL = RMAX, E = C::E, EY = C::EY;
+    using CV = Col8<T>;
+    using V8 = typename CV::V;
+    constexpr int b = C::b, bm = b - 1, NV = C::NV, NS = C::NS, HL = RMAX, LD = C::LD;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    T *rg = reinterpret_cast<T *>(smem_raw);       // [NS][EY][E] (FP32: [NS][EY/2][P2])
-    T *im = rg + NS * C::RG;                        // [NS][EY][IP] (row pitch IP >= b)
-    constexpr int IP = C::IP;
-    const int o1 = items[2 * at.item], o2 = items[2 * at.item + 1];
+    T *s = reinterpret_cast<T *>(smem_raw);         // [NS][EY][LD], planes PL apart
+    __shared__ int nbs[(2 * kMaxWinNr + 2) * (2 * kMaxWinNr + 1)];
+    const int o1 = at.items[2 * at.item], o2 = at.items[2 * at.item + 1];
     const bool pair = o2 >= 0;                      // uniform over the CTA
-    const int ny = pair ? 2 : 1;
     const int rows = pair ? C::EY : C::EY1;         // staged rows per plane
     const int s0 = blockIdx.y * NS;
     const int nd = 2 * nr + 1;
-    const int *nb1 = nbr + (int64_t)o1 * nd * nd;
-    const int *nb2 = pair ? nbr + (int64_t)o2 * nd * nd : nb1;
-    const T *inf = J.in + field * J.in_stride;
-    T *outf = J.out + field * J.out_stride;
+    const int tid = threadIdx.x;
+    // block rows relative to the first output block: -nr .. nr, and nr + 1 of a pair
+    if (tid < (nd + (pair ? 1 : 0)) * nd) {
+        const int dy = tid / nd, dx = tid - dy * nd;
+        nbs[tid] = dy < nd ? at.nbr[(int64_t)o1 * nd * nd + tid] : at.nbr[(int64_t)o2 * nd * nd + (nd - 1) * nd + dx];
+    }
+    __syncthreads();
     // plane-local row -> (z-plane, staged row) with compile-time divisors
     auto split = [&](int row, int &zl, int &yr) {
         zl = pair ? row / C::EY : row / C::EY1;
         yr = row - zl * rows;
     };
     // ---- stage ----
-    // FP64: one staged row per item, layout [NS][EY][E].  FP32: rows 2j and
-    // 2j + 1 per item (the same source block: block edges and the halo are
-    // even), interleaved as [NS][EY/2][E][2] (row pairs P2 apart), so that the
-    // x stencil runs on the packed pair (row 2j, row 2j + 1) with one FP32x2
-    // FMA per weight.
-    constexpr bool PACK = std::is_same<T, float>::value;
-    constexpr int RPI = PACK ? 2 : 1;                  // staged rows per item
-    constexpr int vpr = E / NV;
-    const int total = NS * (rows / RPI) * vpr;
-    constexpr int U = 4;
-    for (int base = threadIdx.x; base < total; base += U * 256) {
-        VT v[U][RPI];
-        int dst[U];
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const int it = base + u * 256;
-            dst[u] = -1;
-#pragma unroll
-            for (int q = 0; q < RPI; ++q) v[u][q] = VT{};
-            if (it >= total) continue;
-            const int rr = it / vpr, cv = it - rr * vpr;
-            int zl, yr;
-            split(rr * RPI, zl, yr);
-            const int ex = cv * NV - HL, ey = yr - HL, z = s0 + zl;
-            dst[u] = PACK ? (zl * (EY / 2) + yr / 2) * C::P2 + cv * NV * 2 : (zl * EY + yr) * E + cv * NV;
-            // block row of ey relative to the first output block: -nr .. ny - 1 + nr
-            const int dyb = (ey + nr * b) >> LB;
-            const int *nbt = dyb <= 2 * nr ? nb1 + dyb * nd : nb2 + (dyb - 1) * nd;
-            const int bi = nbt[(ex + nr * b) >> LB];
-            if (bi >= 0) {
-                const T *src = inf + ((int64_t)bi << (3 * LB)) + (((z << LB) + (ey & bm)) << LB) + (ex & bm);
-#pragma unroll
-                for (int q = 0; q < RPI; ++q) v[u][q] = *reinterpret_cast<const VT *>(src + q * b);
-            }
-        }
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            if (dst[u] < 0) continue;
-            if constexpr (PACK) {
-                const float4 a = v[u][0], c = v[u][RPI - 1];
-                *reinterpret_cast<float4 *>(rg + dst[u]) = make_float4(a.x, c.x, a.y, c.y);
-                *reinterpret_cast<float4 *>(rg + dst[u] + 4) = make_float4(a.z, c.z, a.w, c.w);
-            } else {
-                *reinterpret_cast<VT *>(rg + dst[u]) = v[u][0];
-            }
-        }
+    const T *inf = J.in + at.field * J.in_stride;
+    constexpr int vpr = C::E / NV;
+    for (int it = tid; it < NS * rows * vpr; it += C::THREADS) {
+        const int rr = it / vpr, cv = it - rr * vpr;
+        int zl, yr;
+        split(rr, zl, yr);
+        const int ex = cv * NV - HL, ey = yr - HL;
+        const int bi = nbs[((ey + nr * b) >> LB) * nd + ((ex + nr * b) >> LB)];
+        const T *src = inf + ((int64_t)(bi < 0 ? 0 : bi) << (3 * LB)) + ((((s0 + zl) << LB) + (ey & bm)) << LB) + (ex & bm);
+        async::copy16(s + zl * C::PL + yr * LD + cv * NV, src, bi >= 0);
     }
     WinW<T, RMAX> W;
-    load_weights(W, wg, R);
+    load_weights(W, J.w, J.R);
+    async::copies_done();
     __syncthreads();
-    // ---- x stencil: every staged row, kV outputs per item (two rows in FP32) ----
-    // (Lanes 32 bytes apart in FP32: two-way bank conflicts on these loads.
-    // Mapping the items of a quarter-warp onto distinct bank groups made this
-    // kernel faster alone but the graph step, where it runs beside the FFT
-    // passes, slower, presumably because the shared-memory-bound form leaves
-    // their warps more issue slots.)
-    const int xitems = NS * (rows / RPI) * (b / kV);
-    for (int it = threadIdx.x; it < xitems; it += 256) {
-        const int xv = it % (b / kV);
+    // ---- x stencil ----
+    {
+        constexpr int V = C::V, NIN = V + 2 * RMAX;
         int zl, yr;
-        split(it / (b / kV) * RPI, zl, yr);
-        const int x0 = xv * kV;
-        const int row = zl * EY + yr;
-        // staged x_ext = x0 - HL ...
-        const T *r = PACK ? rg + (zl * (EY / 2) + yr / 2) * C::P2 + 2 * x0 : rg + row * E + x0;
-        if constexpr (PACK) {
-            float2 acc[kV];                                    // (row, row + 1)
+        split(tid / C::GX, zl, yr);
+        const bool on = tid < NS * rows * C::GX;
+        T *row = s + (on ? zl * C::PL + yr * LD : 0) + (tid % C::GX) * V;
+        T in[NIN], acc[V];
+        if (on) {
 #pragma unroll
-            for (int v = 0; v < kV; ++v) acc[v] = make_float2(0.f, 0.f);
-#pragma unroll
-            for (int i = 0; i < (kV + 2 * RMAX) / 2; ++i) {
-                const float4 val = *reinterpret_cast<const float4 *>(r + 4 * i);
-                const float2 pr[2] = {make_float2(val.x, val.y), make_float2(val.z, val.w)};
-#pragma unroll
-                for (int e = 0; e < 2; ++e) {
-                    const int pos = 2 * i + e;
-#pragma unroll
-                    for (int v = 0; v < kV; ++v) {
-                        const int d = pos - HL - v;
-                        if (d >= -RMAX && d <= RMAX) acc[v] = __ffma2_rn(W.w[d < 0 ? -d : d], pr[e], acc[v]);
-                    }
-                }
-            }
-            static_assert(kV == 4, "one float4 per row");
-            *reinterpret_cast<float4 *>(im + row * IP + x0) = make_float4(acc[0].x, acc[1].x, acc[2].x, acc[3].x);
-            *reinterpret_cast<float4 *>(im + (row + 1) * IP + x0) =
-                make_float4(acc[0].y, acc[1].y, acc[2].y, acc[3].y);
-        } else {
-            T acc[kV];
-#pragma unroll
-            for (int v = 0; v < kV; ++v) acc[v] = T(0);
-#pragma unroll
-            for (int i = 0; i < (kV + 2 * RMAX) / NV; ++i) {
-                const VT val = *reinterpret_cast<const VT *>(r + i * NV);
+            for (int i = 0; i < NIN / NV; ++i) {
+                const VT val = *reinterpret_cast<const VT *>(row + i * NV);
                 const T *vs = reinterpret_cast<const T *>(&val);
 #pragma unroll
-                for (int e = 0; e < NV; ++e) {
-                    const int pos = i * NV + e;
+                for (int e = 0; e < NV; ++e) in[i * NV + e] = vs[e];
+            }
+        }
+        if (C::GX > 1) __syncwarp();   // the row's other half is read before this one is overwritten
+        if (on) {
 #pragma unroll
-                    for (int v = 0; v < kV; ++v) {
-                        const int d = pos - HL - v;
-                        if (d >= -RMAX && d <= RMAX) acc[v] += wscalar(W, d < 0 ? -d : d) * vs[e];
-                    }
+            for (int v = 0; v < V; ++v) acc[v] = T(0);
+#pragma unroll
+            for (int pos = 0; pos < NIN; ++pos) {
+#pragma unroll
+                for (int v = 0; v < V; ++v) {
+                    const int d = pos - HL - v;
+                    if (d >= -RMAX && d <= RMAX) acc[v] = fma(wscalar(W, d < 0 ? -d : d), in[pos], acc[v]);
                 }
             }
 #pragma unroll
-            for (int v = 0; v < kV; v += NV) {
+            for (int v = 0; v < V; v += NV) {
                 VT q;
                 T *qq = reinterpret_cast<T *>(&q);
 #pragma unroll
                 for (int e = 0; e < NV; ++e) qq[e] = acc[v + e];
-                *reinterpret_cast<VT *>(im + row * IP + x0 + v) = q;
+                *reinterpret_cast<VT *>(row + v) = q;
             }
         }
     }
     __syncthreads();
-    // ---- y stencil: NV adjacent x, kV consecutive y outputs per item ----
-    const int ypp = ny * (b / kV);                     // y items per plane and x column
-    const int yitems = NS * (b / NV) * ypp;
-    for (int it = threadIdx.x; it < yitems; it += 256) {
-        const int xv = it % (b / NV);
-        const int yv = (it / (b / NV)) % ypp;
-        const int zl = it / ((b / NV) * ypp);
-        const int x = xv * NV, y0 = yv * kV;                  // output row among the ny * b
-        const T *col = im + (zl * EY + y0) * IP + x;          // y_ext = y0 - HL ...
-        VT q[kV];
-        col_window<RMAX>(col, IP, W, q);
-        const int z = s0 + zl;
-        const int o = y0 < b ? o1 : o2;
-        const int yl = y0 & bm;
+    // ---- y stencil: one 8-byte column, VY consecutive outputs per item ----
+    constexpr int XL = b / CV::N, VY = C::VY;
+    T *outf = J.out + at.field * J.out_stride;
+    for (int it = tid; it < XL * NS * C::GY * (pair ? 2 : 1); it += C::THREADS) {
+        const int x = it % XL * CV::N, zl = it / XL % NS, y0 = it / (XL * NS) * VY;
+        const T *col = s + zl * C::PL + y0 * LD + x;          // y_ext = y0 - HL ...
+        V8 acc[VY];
 #pragma unroll
-        for (int v = 0; v < kV; ++v)
-            *reinterpret_cast<VT *>(outf + ((int64_t)o << (3 * LB)) + (((z << LB) + yl + v) << LB) + x) = q[v];
+        for (int v = 0; v < VY; ++v) acc[v] = V8{};
+#pragma unroll
+        for (int pos = 0; pos < VY + 2 * RMAX; ++pos) {
+            const V8 val = *reinterpret_cast<const V8 *>(col + pos * LD);
+#pragma unroll
+            for (int v = 0; v < VY; ++v) {
+                const int d = pos - HL - v;
+                if (d >= -RMAX && d <= RMAX) acc[v] = CV::fma(W.w[d < 0 ? -d : d], val, acc[v]);
+            }
+        }
+        T *dst = outf + ((int64_t)(y0 < b ? o1 : o2) << (3 * LB)) + ((((s0 + zl) << LB) + (y0 & bm)) << LB) + x;
+#pragma unroll
+        for (int v = 0; v < VY; ++v) *reinterpret_cast<V8 *>(dst + (v << LB)) = acc[v];
     }
 }
 
@@ -632,8 +666,8 @@ lgf_status launch_xy_m(lgf_ctx *ctx, int nitems, const SepJobs<T> &jobs, cudaStr
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM);
         if (e != cudaSuccess) return cuda_fail(ctx, e, "cudaFuncSetAttribute");
     }
-    dim3 grid(nitems, C::b / C::NSB, jobs.n * jobs.nf);
-    kern<<<grid, 256, C::SMEM, s>>>(jobs, nbr, items, nr);
+    dim3 grid(nitems, C::b / C::NS, jobs.n * jobs.nf);
+    kern<<<grid, C::THREADS, C::SMEM, s>>>(jobs, nbr, items, nr);
     return LGF_OK;
 }
 
@@ -655,7 +689,6 @@ lgf_status launch_m(lgf_ctx *ctx, int nout, const SepJobs<T> &jobs, cudaStream_t
     using C = Cfg<T, LB, AX>;
     constexpr int b = 1 << LB, E = b + 2 * RMAX;
     constexpr size_t smem = sizeof(T) * (size_t)C::NS * b * E;
-    auto kern = k_sep_win<T, LB, AX, RMAX>;
     // the z pass stages with bulk copies when every job's input is 16-byte
     // aligned (the copies' requirement; block and plane offsets keep it) and
     // the context has a device error word for the bounded waits
@@ -679,12 +712,18 @@ lgf_status launch_m(lgf_ctx *ctx, int nout, const SepJobs<T> &jobs, cudaStream_t
             return LGF_OK;
         }
     }
-    if (smem > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return cuda_fail(ctx, e, "cudaFuncSetAttribute");
+    if constexpr (AX == 2 && LB >= 4) {
+        using Z = ZCfg<T, LB>;
+        k_sep_z<T, LB, RMAX><<<dim3(nout, Z::NY, jobs.n * jobs.nf), Z::THREADS, 0, s>>>(jobs, nbr, nr);
+    } else {
+        auto kern = k_sep_win<T, LB, AX, RMAX>;
+        if (smem > 48 * 1024) {
+            cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            if (e != cudaSuccess) return cuda_fail(ctx, e, "cudaFuncSetAttribute");
+        }
+        dim3 grid(nout, b / C::NS, jobs.n * jobs.nf);
+        kern<<<grid, C::THREADS, smem, s>>>(jobs, nbr, nr);
     }
-    dim3 grid(nout, b / C::NS, jobs.n * jobs.nf);
-    kern<<<grid, C::THREADS, smem, s>>>(jobs, nbr, nr);
     return LGF_OK;
 }
 
@@ -723,24 +762,31 @@ lgf_status launch_xy_rag_m(lgf_ctx *ctx, SepRagJob<T> *jobs, int n, cudaStream_t
         if (e != cudaSuccess) return cuda_fail(ctx, e, "cudaFuncSetAttribute");
     }
     return rag_send_sep<T>(ctx, jobs, n, [&](unsigned gx, const SepRag<T> &t) {
-        kern<<<dim3(gx, C::b / C::NSB, 1), 256, C::SMEM, s>>>(t, nullptr, nullptr, 0);
+        kern<<<dim3(gx, C::b / C::NS, 1), C::THREADS, C::SMEM, s>>>(t, nullptr, nullptr, 0);
     });
 }
 
 template <typename T, int LB, int RMAX>
 lgf_status launch_z_rag_m(lgf_ctx *ctx, SepRagJob<T> *jobs, int n, cudaStream_t s)
 {
-    using C = Cfg<T, LB, 2>;
-    constexpr int b = 1 << LB, E = b + 2 * RMAX;
-    constexpr size_t smem = sizeof(T) * (size_t)C::NS * b * E;
-    auto kern = k_sep_win<T, LB, 2, RMAX, SepRag<T>>;
-    if (smem > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return cuda_fail(ctx, e, "cudaFuncSetAttribute");
+    if constexpr (LB >= 4) {
+        using Z = ZCfg<T, LB>;
+        return rag_send_sep<T>(ctx, jobs, n, [&](unsigned gx, const SepRag<T> &t) {
+            k_sep_z<T, LB, RMAX, SepRag<T>><<<dim3(gx, Z::NY, 1), Z::THREADS, 0, s>>>(t, nullptr, 0);
+        });
+    } else {
+        using C = Cfg<T, LB, 2>;
+        constexpr int b = 1 << LB, E = b + 2 * RMAX;
+        constexpr size_t smem = sizeof(T) * (size_t)C::NS * b * E;
+        auto kern = k_sep_win<T, LB, 2, RMAX, SepRag<T>>;
+        if (smem > 48 * 1024) {
+            cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            if (e != cudaSuccess) return cuda_fail(ctx, e, "cudaFuncSetAttribute");
+        }
+        return rag_send_sep<T>(ctx, jobs, n, [&](unsigned gx, const SepRag<T> &t) {
+            kern<<<dim3(gx, b / C::NS, 1), C::THREADS, smem, s>>>(t, nullptr, 0);
+        });
     }
-    return rag_send_sep<T>(ctx, jobs, n, [&](unsigned gx, const SepRag<T> &t) {
-        kern<<<dim3(gx, b / C::NS, 1), C::THREADS, smem, s>>>(t, nullptr, 0);
-    });
 }
 
 template <typename T, int LB, int AX>
@@ -768,7 +814,7 @@ inline int window_rmax(const SepJobs<T> &jobs, int b, int nr)
     int R = 0;
     for (int i = 0; i < jobs.n; ++i) R = jobs.j[i].R > R ? jobs.j[i].R : R;
     const int rmax = window_class(R);
-    if (rmax == 0 || rmax > nr * b || (b != 8 && b != 16 && b != 32)) return 0;
+    if (rmax == 0 || rmax > nr * b || nr > win::kMaxWinNr || (b != 8 && b != 16 && b != 32)) return 0;
     return rmax;
 }
 

@@ -126,3 +126,18 @@ def test_every_window_class_single_and_paired_blocks(ctx32, ctx64, oracle, prec,
         got = run_intf(ctx, p, alpha)
         assert rel_linf(got, oracle_intf(oracle, p, alpha)) < TOL[prec], (alpha, R)
     assert seen == {4, 8, 12, 16}
+
+
+@pytest.mark.parametrize("prec", ["f32", "f64"])
+@pytest.mark.parametrize("b,seed,extent", [(8, 21, (4, 4, 3)), (16, 22, (1, 4, 1)), (32, 23, (1, 1, 3))])
+def test_every_window_class_more_block_shapes(ctx32, ctx64, oracle, prec, b, seed, extent):
+    """Each radius class on blocks of 8 (windows that reach two neighbours), on
+    a column of blocks in y and on one in z, source and target sets apart from
+    the ragged coincidence of the draw."""
+    ctx = ctx64 if prec == "f64" else ctx32
+    n = int(np.prod(extent))
+    p = li.random_sparse(seed, b=b, nsrc=max(1, n // 2), ntgt=max(2, 2 * n // 3), extent=extent, ncomp=3)
+    for alpha in (0.02, 0.3, 1.0, 2.0) if prec == "f32" else (1e-4, 0.05, 0.25, 0.75):
+        ref = oracle_intf(oracle, p, alpha)
+        if np.abs(ref).max() > 0:
+            assert rel_linf(run_intf(ctx, p, alpha), ref) < TOL[prec], alpha
