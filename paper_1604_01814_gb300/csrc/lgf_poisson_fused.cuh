@@ -232,7 +232,7 @@ __global__ void __cluster_dims__(NCL, 1, 1) __launch_bounds__(YXCfg<MY, MX>::THR
         const Cx<T> *plane = J.B + field * g.Bstride + (int64_t)zi * MY * g.ld;
         const bool half = lo + n <= MY / 2;
         constexpr int RL = PY::RL, R0 = PY::R0;
-        constexpr int NGL = PY::GL / PY::TPC;
+        constexpr int NGL = PY::NGL;
         const int64_t istep = (int64_t)(MY / RL) * g.ld;
         const int ntile = (K + W - 1) / W;
 #pragma unroll 1
@@ -244,6 +244,7 @@ __global__ void __cluster_dims__(NCL, 1, 1) __launch_bounds__(YXCfg<MY, MX>::THR
 #pragma unroll
             for (int i = 0; i < NGL; ++i) {
                 const int gg = t + i * PY::TPC;
+                if (PY::MASKL && gg >= PY::GL) break;
                 int64_t off = (int64_t)freq_of<MY>(gg * RL) * g.ld;
 #pragma unroll
                 for (int q = 0; q < RL; ++q) {
@@ -255,6 +256,7 @@ __global__ void __cluster_dims__(NCL, 1, 1) __launch_bounds__(YXCfg<MY, MX>::THR
 #pragma unroll
                 for (int i = 0; i < NGL; ++i) {
                     const int gg = t + i * PY::TPC;
+                    if (PY::MASKL && gg >= PY::GL) break;
                     Dft<RL, 1, T>::run(cc[i]);
 #pragma unroll
                     for (int q = 0; q < RL; ++q) s[ad(w, (gg * RL) + q)] = cc[i][q];

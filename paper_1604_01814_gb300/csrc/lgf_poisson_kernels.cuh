@@ -24,34 +24,39 @@ namespace pk {
 constexpr int cgcd(int a, int b) { return b == 0 ? a : cgcd(b, a % b); }
 
 // Stage plan of a length M (2^k, 3 * 2^k or 5 * 2^k, 32..4096): a first stage
-// of radix R0, for M >= 512 and most 3 * 2^k, 5 * 2^k a middle stage of radix
-// R1 (R0, R1 powers of two; the middle stage keeps more threads per line),
-// and a last stage of radix RL (16, 8 or 4; 12 when M = 3 * 2^k, 20 when
-// M = 5 * 2^k).  Every stage
-// before the last splits off a power of two, so its twiddle index stays
-// j q M/N with M/N a power of two.  TPC threads share a line: the greatest
-// common divisor of the stages' group counts, so that every thread owns a
-// whole number of groups in every stage.
+// of radix R0, for M >= 384 a middle stage of radix R1 (R0, R1 powers of two),
+// and a last stage of even radix RL.  Every stage before the last splits off
+// a power of two, so its twiddle index stays j q M/N with M/N a power of two.
+// TPC threads share a line.  In the three-stage plans it is the greatest common
+// divisor of the stages' group counts, so that every thread owns a whole number of
+// groups in every stage; the two-stage plans have one group per thread in the
+// longer stage, and the threads past the shorter stage's groups (whole warps,
+// as lanes run along columns) sit it out.
+// Lengths 96, 192 and 320 had three stages (4 x 2 x 12, 4 x 4 x 12, 4 x 4 x 20), 80 and
+// 160 a radix of 20: with two stages half the shared-memory passes and barriers go,
+// and more of the butterflies are packed.  z pass at length 320 (refresh of 556 blocks)
+// 315 -> 297 us, the refresh 660 -> 631 us, the 64-plate batch 3.96 -> 3.89 ms.
 template <int ML>
 struct Plan {
     static constexpr int M = ML;
-    static constexpr int R0 = M == 80 || M == 96 || M == 192 || M == 320 ? 4
-                            : M == 32 || M == 64 || M == 160 || M == 384 || M == 512 || M == 640 || M == 768 ||
+    static constexpr int R0 = M == 32 || M == 64 || M == 80 || M == 96 || M == 384 || M == 512 || M == 640 || M == 768 ||
                                       M == 1280
                                   ? 8
                                   : 16;
-    static constexpr int R1 = M == 96 ? 2
-                            : M == 192 || M == 320 || M == 384 || M == 640 ? 4
+    static constexpr int R1 = M == 384 || M == 640 ? 4
                             : M == 512 || M == 768 || M == 1024 || M == 1280 || M == 1536 || M == 2560 ? 8
                             : M == 2048 || M == 3072 || M == 4096 ? 16 : 1;
     static constexpr int RL = M / (R0 * R1);
     static constexpr int NST = R1 > 1 ? 3 : 2;
     static constexpr int N1 = M / R0;                             // sub-problem size entering stage 1
     static constexpr int G0 = M / R0, G1 = M / R1, GL = M / RL;   // groups per stage
-    static constexpr int TPC = cgcd(cgcd(G0, NST == 3 ? G1 : G0), GL);
+    static constexpr int TPC = NST == 3 ? cgcd(cgcd(G0, G1), GL) : cgcd(G0, GL) > 4 || M == 32 ? cgcd(G0, GL)
+                                                                 : G0 > GL ? G0 : GL;
+    static constexpr int NG0 = (G0 + TPC - 1) / TPC, NGL = (GL + TPC - 1) / TPC;   // rounds of groups
+    static constexpr bool MASK0 = G0 % TPC != 0, MASKL = GL % TPC != 0;            // the last round is partial
     static constexpr int TW1 = (R0 - 1) * G0;                     // first twiddle of the middle stage
-    static_assert(R0 * R1 * RL == M && RL <= 20 && RL >= 4, "plan must cover the length");
-    static_assert(G0 % TPC == 0 && G1 % TPC == 0 && GL % TPC == 0, "whole groups per thread");
+    static_assert(R0 * R1 * RL == M && RL <= 20 && RL >= 4 && RL % 2 == 0, "plan must cover the length");
+    static_assert(NST == 2 || (G0 % TPC == 0 && G1 % TPC == 0 && GL % TPC == 0), "whole groups per thread");
 };
 
 // Position of frequency k after the forward sweep, and back: position
@@ -263,7 +268,7 @@ __device__ __forceinline__ void col_forward_body(int bx, int by, const Cx<T> *__
     Cx<T> *ob = out + by * out_field + pl * out_plane + kx;
     const ColAddrW ad{W};
     constexpr int R0 = P::R0;
-    constexpr int NG0 = P::G0 / P::TPC;
+    constexpr int NG0 = P::NG0;
     constexpr int NP = HALF ? R0 / 2 : R0;
     const int64_t istep = (int64_t)P::G0 * rs;
     Cx<T> a[NG0][R0];
@@ -274,7 +279,7 @@ __device__ __forceinline__ void col_forward_body(int bx, int by, const Cx<T> *__
             const Cx<T> *src = ib + (int64_t)r * rs;
 #pragma unroll
             for (int p = 0; p < NP; ++p) {
-                const bool ok = live && (unsigned)(r + p * P::G0) < (unsigned)n;
+                const bool ok = live && (unsigned)(r + p * P::G0) < (unsigned)n && (!P::MASK0 || t + i * P::TPC < P::G0);
                 a[i][p] = ok ? *src : Cx<T>{T(0), T(0)};
                 src += istep;
             }
@@ -288,7 +293,8 @@ __device__ __forceinline__ void col_forward_body(int bx, int by, const Cx<T> *__
 #pragma unroll
             for (int p = 0; p < NP; ++p) {
                 const int y = r + p * P::G0;
-                const bool ok = live && (unsigned)y < (unsigned)n && rf.row(pm, y);
+                const bool ok =
+                    live && (unsigned)y < (unsigned)n && rf.row(pm, y) && (!P::MASK0 || t + i * P::TPC < P::G0);
                 a[i][p] = ok ? *src : Cx<T>{T(0), T(0)};
                 src += istep;
             }
@@ -298,6 +304,7 @@ __device__ __forceinline__ void col_forward_body(int bx, int by, const Cx<T> *__
 #pragma unroll
     for (int i = 0; i < NG0; ++i) {
         const int g = t + i * P::TPC;
+        if (P::MASK0 && g >= P::G0) break;
         dif_group<P::R0, P::G0, HALF>(a[i], g, tw);
 #pragma unroll
         for (int q = 0; q < R0; ++q) s[ad(w, q * P::G0 + g)] = a[i][q];
@@ -361,12 +368,13 @@ __device__ __forceinline__ void col_inverse_body(int bx, int by, const Cx<T> *__
     Cx<T> *ob = out + by * out_field + pl * out_plane + kx;
     const ColAddrW ad{W};
     constexpr int RL = P::RL;
-    constexpr int NGL = P::GL / P::TPC;
+    constexpr int NGL = P::NGL;
     const int64_t istep = (int64_t)(M / RL) * rs;
     Cx<T> c[NGL][RL];
 #pragma unroll
     for (int i = 0; i < NGL; ++i) {
         const int g = t + i * P::TPC;
+        if (P::MASKL && g >= P::GL) break;
         const Cx<T> *src = ib + (int64_t)freq_of<ML>(g * P::RL) * rs;
 #pragma unroll
         for (int q = 0; q < RL; ++q) {
@@ -377,6 +385,7 @@ __device__ __forceinline__ void col_inverse_body(int bx, int by, const Cx<T> *__
 #pragma unroll
     for (int i = 0; i < NGL; ++i) {
         const int g = t + i * P::TPC;
+        if (P::MASKL && g >= P::GL) break;
         Dft<RL, 1, T>::run(c[i]);
 #pragma unroll
         for (int q = 0; q < RL; ++q) s[ad(w, (g * P::RL) + q)] = c[i][q];
@@ -433,7 +442,7 @@ __global__ void __launch_bounds__(W * Plan<ML>::TPC) k_col_inverse(const Cx<T> *
 // leaves the choice to the compiler: 4 up to length 192, 3 above).
 template <typename T, int ML, int ZV = 0>
 struct ConvOcc {
-    static constexpr int base = sizeof(T) == 4 ? (ML == 256 ? 4 : ML == 320 || ML == 384 || ML == 512 ? 3 : ML == 640 || ML == 1536 || ML == 2560 || ML == 3072 ? 2 : 1) : 1;
+    static constexpr int base = sizeof(T) == 4 ? (ML == 160 || ML == 192 || ML == 256 ? 4 : ML == 320 || ML == 384 || ML == 512 ? 3 : ML == 640 || ML == 1536 || ML == 2560 || ML == 3072 ? 2 : 1) : 1;
     static constexpr int value = ZV == 0 ? base : (base == 1 ? (ML <= 192 ? 4 : 3) : base + 1);
 };
 
@@ -462,7 +471,7 @@ __device__ __forceinline__ void col_convolve_body(int bx, int nf, Cx<T> *__restr
     Cx<T> *bb = B + field_i * field + (int64_t)ky * ld + kx;
     const ColAddrW ad{W};
     constexpr int R0 = P::R0;
-    constexpr int NG0 = P::G0 / P::TPC;
+    constexpr int NG0 = P::NG0;
     const int64_t step0 = (int64_t)P::G0 * plane;
     {
         Cx<T> a[NG0][R0];
@@ -472,7 +481,7 @@ __device__ __forceinline__ void col_convolve_body(int bx, int nf, Cx<T> *__restr
             const Cx<T> *src = bb + (int64_t)r * plane;
 #pragma unroll
             for (int p = 0; p < R0 / 2; ++p) {
-                const bool ok = live && (unsigned)(r + p * P::G0) < (unsigned)ns;
+                const bool ok = live && (unsigned)(r + p * P::G0) < (unsigned)ns && (!P::MASK0 || t + i * P::TPC < P::G0);
                 a[i][p] = ok ? *src : Cx<T>{T(0), T(0)};
                 src += step0;
             }
@@ -481,6 +490,7 @@ __device__ __forceinline__ void col_convolve_body(int bx, int nf, Cx<T> *__restr
 #pragma unroll
         for (int i = 0; i < NG0; ++i) {
             const int g = t + i * P::TPC;
+            if (P::MASK0 && g >= P::G0) break;
             dif_group<P::R0, P::G0, true>(a[i], g, tw);
 #pragma unroll
             for (int q = 0; q < R0; ++q) s[ad(w, q * P::G0 + g)] = a[i][q];
@@ -593,32 +603,29 @@ struct RowLay {
     // threads per line: 16 to 24 values each (a masked last round where TPC
     // does not divide the first stage's groups); TPC is a multiple of R0 in the
     // three-stage plans
-    static constexpr int TPC = ML <= 32 || ML == 80 ? 4
+    static constexpr int TPC = ML <= 32 ? 4
                              : ML <= 160 ? 8
+                             : ML == 320 ? 20
                              : ML <= 384 ? 16
                              : ML <= 768 || ML == 1280 ? 32
                              : ML == 2048 || ML == 4096 ? 128
                                          : 64;
-    // lines per CTA: 8 up to length 768 (16 for the plans that start with radix 4,
-    // whose 8-line layout would meet conflicts; 32 for the shortest lines, which would
-    // leave a CTA of two warps), 4 above, so that several CTAs of an SM
-    // overlap their loads, stages and stores and a small box still fills the GPU: 16
-    // lines at length 256 took the 128^3 box's batch from 99.7 to 105.3 us, 8 lines
+    // lines per CTA: 8 up to length 768 (32 for the shortest lines, which would
+    // leave a CTA of one warp), 4 above, so that several CTAs of an SM overlap
+    // their loads, stages and stores and a small box still fills the GPU: 16 lines at
+    // length 256 took the 128^3 box's batch from 99.7 to 105.3 us, 8 lines
     // at length 1024 the wake's x forward from 648 to 804 us
     static constexpr int SIZE = int(sizeof(Cx<T>));
     static constexpr bool fit(int l) { return (ML * (l + 1) + 64 + ML) * SIZE <= 112 * 1024; }
     static constexpr int LPC = TPC == 4 ? 32
-                             : ML <= 768 && P::R0 < 8 && fit(16) ? 16
                              : (ML <= 768 || ML == 1280) && fit(8) ? 8
                              : fit(4) ? 4 : ML * SIZE <= 48 * 1024 ? 2 : 1;
     static constexpr int LD = LPC > 1 ? LPC + 1 : 1;
-    static constexpr bool FEW = LPC < 16 && P::R0 >= 8;
-    static constexpr int C1 = FEW ? LPC : P::R0 == 16 ? 1
-                            : P::R0 == 8 ? (P::NST == 2 ? 2 : 1)
-                            : P::NST == 2 ? 4 : ML == 96 ? 2 : 1;
-    static constexpr int SH = FEW ? (LPC == 8 ? 1 : LPC == 4 ? 2 : 3) : P::R0 == 16 ? 4
-                            : P::R0 == 8 ? (P::NST == 2 || P::RL == 8 ? 3 : 2)
-                            : ML == 96 ? 1 : 2;
+    static constexpr bool FEW = LPC < 16;
+    static constexpr int C1 = FEW ? LPC : P::R0 == 16 ? 1 : P::NST == 2 ? 2 : 1;
+    static constexpr int SH = FEW ? (LPC == 8 ? 1 : LPC == 4 ? 2 : 3)
+                            : P::R0 == 16 ? 4
+                            : P::NST == 2 || P::RL == 8 ? 3 : 2;
     static constexpr int S1 = congruent(P::N1 * LD, C1);
     static constexpr int S2 = congruent(((1 << SH) - 1) * S1 + P::N1 * LD, FEW ? 1 : 8);
     static __host__ __device__ constexpr int base(int q0) { return (q0 & ((1 << SH) - 1)) * S1 + (q0 >> SH) * S2; }
@@ -1011,7 +1018,7 @@ __global__ void __launch_bounds__(W * Plan<ML>::TPC, ConvOcc<T, ML, ZV>::value) 
 template <typename T, int ML>
 struct ColCfg {
     static constexpr int TPC = Plan<ML>::TPC;
-    static constexpr int W0 = 256 / TPC < 8 ? 8 : (256 / TPC > 32 ? 32 : 256 / TPC);
+    static constexpr int W0 = TPC <= 8 ? 32 : TPC <= 20 ? 16 : 8;
     static constexpr int WMAX = int(98304 / (sizeof(Cx<T>) * ML)) < 1 ? 1 : int(98304 / (sizeof(Cx<T>) * ML));
     static constexpr int W = W0 < WMAX ? W0 : WMAX;
     static constexpr size_t SMEM = sizeof(Cx<T>) * (((size_t)ML) * (W + 1));
