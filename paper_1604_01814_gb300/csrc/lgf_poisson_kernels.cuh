@@ -50,8 +50,9 @@ struct Plan {
     static constexpr int NST = R1 > 1 ? 3 : 2;
     static constexpr int N1 = M / R0;                             // sub-problem size entering stage 1
     static constexpr int G0 = M / R0, G1 = M / R1, GL = M / RL;   // groups per stage
-    static constexpr int TPC = NST == 3 ? cgcd(cgcd(G0, G1), GL) : cgcd(G0, GL) > 4 || M == 32 ? cgcd(G0, GL)
-                                                                 : G0 > GL ? G0 : GL;
+    static constexpr int TPC = NST == 3 ? cgcd(cgcd(G0, G1), GL)
+                             : cgcd(G0, GL) <= 4 && M != 32 ? (G0 > GL ? G0 : GL)
+                                                                         : cgcd(G0, GL);
     static constexpr int NG0 = (G0 + TPC - 1) / TPC, NGL = (GL + TPC - 1) / TPC;   // rounds of groups
     static constexpr bool MASK0 = G0 % TPC != 0, MASKL = GL % TPC != 0;            // the last round is partial
     static constexpr int TW1 = (R0 - 1) * G0;                     // first twiddle of the middle stage
@@ -442,7 +443,7 @@ __global__ void __launch_bounds__(W * Plan<ML>::TPC) k_col_inverse(const Cx<T> *
 // leaves the choice to the compiler: 4 up to length 192, 3 above).
 template <typename T, int ML, int ZV = 0>
 struct ConvOcc {
-    static constexpr int base = sizeof(T) == 4 ? (ML == 160 || ML == 192 || ML == 256 ? 4 : ML == 320 || ML == 384 || ML == 512 ? 3 : ML == 640 || ML == 1536 || ML == 2560 || ML == 3072 ? 2 : 1) : 1;
+    static constexpr int base = sizeof(T) == 4 ? (ML == 160 || ML == 192 || ML == 256 ? 4 : ML == 320 ? 5 : ML == 384 || ML == 512 ? 3 : ML == 640 || ML == 1536 || ML == 2560 || ML == 3072 ? 2 : 1) : 1;
     static constexpr int value = ZV == 0 ? base : (base == 1 ? (ML <= 192 ? 4 : 3) : base + 1);
 };
 
@@ -1024,6 +1025,16 @@ struct ColCfg {
     static constexpr size_t SMEM = sizeof(Cx<T>) * (((size_t)ML) * (W + 1));
 };
 
+// The z pass's width: 8 columns at length 320, where five CTAs of 160 threads keep
+// their 72 registers (three of 320 had 64 and spilled: 295 against 283 us for the
+// refresh of 556 blocks).  Elsewhere the column passes' width: 8 columns at 192, 256
+// and 384 took the sphere Poisson apply from 152.4 to 156.6 us and the
+// 512x256x256 wake from 6.10 to 7.18 ms.
+template <typename T, int ML>
+struct ConvCfg : ColCfg<T, ML> {
+    static constexpr int W = ML == 320 ? 8 : ColCfg<T, ML>::W;
+    static constexpr size_t SMEM = sizeof(Cx<T>) * (((size_t)ML) * (W + 1));
+};
 }  // namespace pk
 
 // Launch entry points (one set per precision, instantiated in
@@ -1170,7 +1181,7 @@ template <typename T, int ML, int SPEC>
 lgf_status col_convolve_m(lgf_ctx *ctx, const PoissonGeom &g, Cx<T> *B, const T *spec, const Cx<T> *tw, int nfields,
                           cudaStream_t s)
 {
-    using C = ColCfg<T, ML>;
+    using C = ConvCfg<T, ML>;
     // the register variant is an FP32 choice (FP64 runs one CTA per SM)
     auto kern = (sizeof(T) == 4 && g.zvar) ? k_col_convolve<T, ML, C::W, SPEC, sizeof(T) == 4 ? 1 : 0>
                                            : k_col_convolve<T, ML, C::W, SPEC, 0>;
@@ -1282,7 +1293,7 @@ lgf_status col_inverse_rag_m(lgf_ctx *ctx, bool half_out, ColJob<T> *jobs, int n
 template <typename T, int ML, int SPEC>
 lgf_status col_convolve_rag_m(lgf_ctx *ctx, int zvar, ConvJob<T> *jobs, int n, cudaStream_t s)
 {
-    using C = ColCfg<T, ML>;
+    using C = ConvCfg<T, ML>;
     auto kern = (sizeof(T) == 4 && zvar) ? k_col_convolve_rag<T, ML, C::W, SPEC, sizeof(T) == 4 ? 1 : 0>
                                          : k_col_convolve_rag<T, ML, C::W, SPEC, 0>;
     for (int i = 0; i < n; ++i) {
