@@ -618,7 +618,8 @@ struct RowLay {
     // at length 1024 the wake's x forward from 648 to 804 us
     static constexpr int SIZE = int(sizeof(Cx<T>));
     static constexpr bool fit(int l) { return (ML * (l + 1) + 64 + ML) * SIZE <= 112 * 1024; }
-    static constexpr int LPC = TPC == 4 ? 32
+    static constexpr int LPC = sizeof(T) == 8 && ML <= 128 ? 4   // (FP64: every SM needs lines)
+                             : TPC == 4 ? 32
                              : (ML <= 768 || ML == 1280) && fit(8) ? 8
                              : fit(4) ? 4 : ML * SIZE <= 48 * 1024 ? 2 : 1;
     static constexpr int LD = LPC > 1 ? LPC + 1 : 1;
@@ -1019,7 +1020,11 @@ __global__ void __launch_bounds__(W * Plan<ML>::TPC, ConvOcc<T, ML, ZV>::value) 
 template <typename T, int ML>
 struct ColCfg {
     static constexpr int TPC = Plan<ML>::TPC;
-    static constexpr int W0 = TPC <= 8 ? 32 : TPC <= 20 ? 16 : 8;
+    // FP64 runs at two lanes a clock and SM: what counts is that every SM has
+    // columns, not how many CTAs share one.  With 32 columns a CTA the 32^3 box (length
+    // 64) had 33 CTAs in the y passes and 66 in z: 72.6 us, now 51.2; the FP64 sphere
+    // Poisson apply 3623 -> 3548 us
+    static constexpr int W0 = sizeof(T) == 8 ? 8 : TPC <= 8 ? 32 : TPC <= 20 ? 16 : 8;
     static constexpr int WMAX = int(98304 / (sizeof(Cx<T>) * ML)) < 1 ? 1 : int(98304 / (sizeof(Cx<T>) * ML));
     static constexpr int W = W0 < WMAX ? W0 : WMAX;
     static constexpr size_t SMEM = sizeof(Cx<T>) * (((size_t)ML) * (W + 1));
