@@ -351,6 +351,31 @@ struct IntfGroupRef {
 lgf_status intf_ragged_scratch(lgf_ctx *ctx, const IntfGroupRef *gs, int n, Scratch *sc);
 lgf_status intf_run_ragged(lgf_ctx *ctx, const IntfGroupRef *gs, int n, cudaStream_t s, Scratch *sc);
 
+// The cells one thread of a staggered stencil kernel takes along x: 16 bytes of
+// a row, or one cell where a field is off the 16-byte alignment.
+template <typename T, bool VEC>
+struct CellVec {
+    using V = T;
+};
+template <>
+struct CellVec<float, true> {
+    using V = float4;
+};
+template <>
+struct CellVec<double, true> {
+    using V = double2;
+};
+inline bool cells_aligned(const void *a, const void *b, const void *c)
+{
+    return ((reinterpret_cast<uintptr_t>(a) | reinterpret_cast<uintptr_t>(b) | reinterpret_cast<uintptr_t>(c)) & 15) == 0;
+}
+template <typename T, bool VEC>
+unsigned cell_grid(int64_t ncell)   // CTAs of 256 threads
+{
+    constexpr int64_t per = 256 * sizeof(typename CellVec<T, VEC>::V) / sizeof(T);
+    return (unsigned)((ncell + per - 1) / per);
+}
+
 // Curl and velocity refresh (lgf_curl.cu)
 lgf_status curl_plan(lgf_ctx *ctx, const lgf_blockset *src, const lgf_blockset *tgt, int dir, CurlPlan **out);
 lgf_status curl_run(lgf_ctx *ctx, const CurlPlan *pl, const void *in, void *out, int nrhs, double scale,

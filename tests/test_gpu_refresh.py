@@ -107,3 +107,20 @@ def test_velocity_refresh_multiple_rhs_equal_single(ctx32):
         ctx32.velocity_refresh(b, src, tgt, u[r * n_in:(r + 1) * n_in].contiguous(), one)
         torch.cuda.synchronize()
         assert torch.equal(one, both[r * n_out:(r + 1) * n_out])
+
+
+@pytest.mark.parametrize("prec", ["f64", "f32"])
+@pytest.mark.parametrize("adjoint", [False, True])
+@pytest.mark.parametrize("b", [4, 8, 16, 32, 64])
+def test_curl_on_and_off_the_vector_alignment(prec, adjoint, b, ctx64, ctx32):
+    """Fields one value off the 16-byte alignment take one cell per thread,
+    aligned ones 16 bytes of a row: the same bits on every block edge."""
+    ctx = ctx64 if prec == "f64" else ctx32
+    src, tgt = _sets(5, b, 2, 3, (2, 2, 1))
+    gen = torch.Generator("cuda").manual_seed(b)
+    a = torch.randn(3 * src.shape[0] * b ** 3 + 1, dtype=ctx.dtype, device="cuda", generator=gen)
+    run = ctx.curl_adjoint if adjoint else ctx.curl
+    out = [torch.full((3 * tgt.shape[0] * b ** 3 + 1,), float("nan"), dtype=ctx.dtype, device="cuda") for _ in range(2)]
+    run(b, src, tgt, a[1:], out[0][1:])
+    run(b, src, tgt, a[1:].clone(), out[1][:-1])
+    assert torch.equal(out[0][1:], out[1][:-1])

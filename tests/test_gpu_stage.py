@@ -117,3 +117,16 @@ def test_stage_force_product_sizes(prec, nm, shift, ctx64, ctx32):
         bound += w.abs().T @ (w.abs() @ ub.double().abs())
     tol = 4 * (n + 2) * torch.finfo(dt).eps / 2
     assert bool(((f.double() - ref).abs() <= tol * bound).all())
+
+
+@pytest.mark.parametrize("prec", ["f64", "f32"])
+@pytest.mark.parametrize("b", [4, 8, 16])
+def test_stage_right_hand_side_off_the_vector_alignment(prec, b, ctx64, ctx32):
+    """r one value off the 16-byte alignment: the same bits as aligned."""
+    ctx = ctx64 if prec == "f64" else ctx32
+    D = li.random_sparse(9, b=b, nsrc=5, ntgt=1, extent=(3, 2, 2)).src
+    r = torch.randn(3 * D.shape[0] * b ** 3 + 1, dtype=ctx.dtype, device="cuda")
+    u = [torch.empty(3 * D.shape[0] * b ** 3, dtype=ctx.dtype, device="cuda") for _ in range(2)]
+    ctx.nested_projection_stage(b, D, r[1:], u[0], alpha=0.1)
+    ctx.nested_projection_stage(b, D, r[1:].clone(), u[1], alpha=0.1)
+    assert torch.equal(u[0], u[1])
