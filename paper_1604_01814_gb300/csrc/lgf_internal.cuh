@@ -49,12 +49,13 @@ struct PoissonGeom {
     int64_t Astride;    // complex elements per field in scratch A
     int64_t Bstride;    // complex elements per field in scratch B
     int ldA_y;          // rows per z-plane in A (max(Ls_y, Lt_y))
-    // embedding along x and y: 0 = even (M >= 2L - 1 on the union extent,
-    // real spectrum along that axis); 1 = shifted window (M >= Ls + Lt - 1,
+    // embedding per axis: 0 = even (M >= 2L - 1 on the union extent, real
+    // spectrum along that axis); 1 = shifted window (M >= Ls + Lt - 1,
     // source and target both placed at 0, complex spectrum):
-    // h[m] = G_L(m + c) for m < P, G_L(m - M + c) above.  z is always even.
+    // h[m] = G_L(m + c) for m < P, G_L(m - M + c) above.
     int xasym, xc, xP;
     int yasym, yc, yP;
+    int zasym, zc, zP;
     int zvar;           // z-pass variant: 0 default, 1 one more CTA per SM (tighter register cap)
     int fuse;           // FP32: the y and x inverses as one cluster kernel where available
     double scale;       // dx^2
@@ -119,8 +120,10 @@ struct Spectrum {
     double alpha = 0.0;       // 0: G_L; > 0: G_K(alpha)
     int xasym = 0, xc = 0, xP = 0;   // the x and y embeddings of PoissonGeom
     int yasym = 0, yc = 0, yP = 0;
-    // (Mz/2+1)(My/2+1)(Mx/2+1) values, context precision, scaled by
-    // 1/(MxMyMz): reals for the even x embedding, complex for the shifted one
+    int zasym = 0, zc = 0, zP = 0;
+    // (Mz/2+1)(My/2+1)(Mx/2+1) values (all ky or kz of a window shifted in y or
+    // z), context precision, scaled by 1/(MxMyMz): reals when every axis is
+    // even, complex otherwise
     void *dev = nullptr;
     uint64_t used = 0;
     Spectrum() = default;
@@ -278,8 +281,7 @@ lgf_status table_build(lgf_ctx *ctx, int radius, cudaStream_t s);
 lgf_status gk_table(lgf_ctx *ctx, double alpha, const double **out, cudaStream_t s);
 lgf_status table_lookup(lgf_ctx *ctx, const double *table, const int32_t *off, int64_t n, double *out,
                         cudaStream_t s);
-lgf_status kernel_window(lgf_ctx *ctx, const double *table, const int M[3], int xc, int xP, int yc, int yP,
-                         double *box, cudaStream_t s);
+lgf_status kernel_window(lgf_ctx *ctx, const double *table, const PoissonGeom &g, double *box, cudaStream_t s);
 lgf_status bessel_weights(lgf_ctx *ctx, double z, int nmax, double *out_dev, cudaStream_t s);
 // FP64 direct sums dx^2 sum_m G_L(t - m) f(m) of one source field at npts
 // lattice points (host [npts][3]); values to host out.  Synchronous.

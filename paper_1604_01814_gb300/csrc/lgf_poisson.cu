@@ -47,6 +47,8 @@ namespace lgf {
                                                          const Cx<T> *, int, cudaStream_t);                      \
     extern template lgf_status launch_col_convolve<T, 2>(lgf_ctx *, const PoissonGeom &, Cx<T> *, const T *,   \
                                                          const Cx<T> *, int, cudaStream_t);                      \
+    extern template lgf_status launch_col_convolve<T, 3>(lgf_ctx *, const PoissonGeom &, Cx<T> *, const T *,   \
+                                                         const Cx<T> *, int, cudaStream_t);                      \
     extern template lgf_status launch_row_forward_rag<T>(lgf_ctx *, int, pk::RowJob<T> *, int, cudaStream_t);    \
     extern template lgf_status launch_row_inverse_rag<T>(lgf_ctx *, int, bool, pk::RowJob<T> *, int,             \
                                                          cudaStream_t);                                          \
@@ -58,6 +60,8 @@ namespace lgf {
     extern template lgf_status launch_col_convolve_rag<T, 1>(lgf_ctx *, int, int, pk::ConvJob<T> *, int,         \
                                                              cudaStream_t);                                      \
     extern template lgf_status launch_col_convolve_rag<T, 2>(lgf_ctx *, int, int, pk::ConvJob<T> *, int,         \
+                                                             cudaStream_t);                                      \
+    extern template lgf_status launch_col_convolve_rag<T, 3>(lgf_ctx *, int, int, pk::ConvJob<T> *, int,         \
                                                              cudaStream_t);
 LGF_EXTERN_PASSES(float)
 LGF_EXTERN_PASSES(double)
@@ -108,6 +112,7 @@ bool poisson_geometry(const PoissonPlan &pl, const PoissonChoice &ch, PoissonGeo
     PoissonGeom &g = *gp;
     const int b = pl.b;
     g.b = b;
+    g.zasym = 0;
     for (int d = 0; d < 3; ++d) {
         const int lo = std::min(pl.slo[d], pl.tlo[d]), hi = std::max(pl.shi[d], pl.thi[d]);
         const int64_t L = ((int64_t)hi - lo + 1) * b;
@@ -115,7 +120,15 @@ bool poisson_geometry(const PoissonPlan &pl, const PoissonChoice &ch, PoissonGeo
         g.Lt[d] = (pl.thi[d] - pl.tlo[d] + 1) * b;
         g.nbs[d] = pl.shi[d] - pl.slo[d] + 1;
         g.nbt[d] = pl.thi[d] - pl.tlo[d] + 1;
-        const bool shift = d < 2 && ch.shift[d];
+        bool shift = d < 2 && ch.shift[d];
+        if (d == 2 && (ch.shift[0] || ch.shift[1])) {
+            // z follows x and y: shifted where that is shorter.  Its spectrum has all kz
+            // (twice the values of one shifted in x or y, which is complex
+            // already; an even one would grow from a real half, so z alone stays even)
+            const int Ms = fft_size_bumped(g.Ls[2] + g.Lt[2] - 1, ch.bump[2]);
+            shift = 2 * g.Ls[2] <= Ms && Ms <= kMaxFft && Ms < fft_size_bumped((int)std::min<int64_t>(2 * L - 1, 2 * kMaxFft), ch.bump[2]);
+            g.zasym = shift;
+        }
         if (!shift) {
             // even embedding on the union extent: every offset within +-(L - 1)
             if (L > kMaxFft / 2) return false;
@@ -138,6 +151,8 @@ bool poisson_geometry(const PoissonPlan &pl, const PoissonChoice &ch, PoissonGeo
     g.yasym = ch.shift[1];
     g.yc = ch.shift[1] ? (pl.tlo[1] - pl.slo[1]) * b : 0;
     g.yP = ch.shift[1] ? g.Lt[1] + (g.M[1] - g.Ls[1] + 1 - g.Lt[1]) / 2 : g.M[1] / 2;
+    g.zc = g.zasym ? (pl.tlo[2] - pl.slo[2]) * b : 0;
+    g.zP = g.zasym ? g.Lt[2] + (g.M[2] - g.Ls[2] + 1 - g.Lt[2]) / 2 : g.M[2] / 2;
     g.zvar = ch.zvar;
     g.fuse = ch.fuse;
     g.Kx = g.M[0] / 2 + 1;
@@ -218,12 +233,12 @@ lgf_status twiddle_exponents(lgf_ctx *ctx, int M, std::vector<int> *e)
 
 // Spectrum of a shifted window: the complex forward transform at
 // kx <= Mx/2, ky < nky (My/2 + 1 when the window is even in y, My when it
-// is shifted in y), kz <= Mz/2 (even in z), scaled by 1/(Mx My Mz).
+// is shifted in y), kz < nkz (Mz/2 + 1 or Mz likewise), scaled by 1/(Mx My Mz).
 template <typename T>
 __global__ void k_extract_c(const Cx<double> *__restrict__ B, Cx<T> *__restrict__ spec, int Mx, int My, int Mz,
-                            int nky, int ld)
+                            int nky, int nkz, int ld)
 {
-    const int K = Mx / 2 + 1, Khy = nky, Khz = Mz / 2 + 1;
+    const int K = Mx / 2 + 1, Khy = nky, Khz = nkz;
     const int64_t n = (int64_t)K * Khy * Khz;
     const double sc = 1.0 / ((double)Mx * My * Mz);
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
@@ -328,8 +343,9 @@ lgf_status run_passes(lgf_ctx *ctx, const PoissonGeom &g, const T *f, T *u, Cx<T
     if (spectrum_mode)
         return launch_col_forward<T>(ctx, Mz, K, My, nf, B, B, 0, Mz, planeB, planeB, ld, ld, g.Bstride, g.Bstride, twz,
                                      pk::RowFlags{}, s, "spectrum_z_forward");
-    // the z pass for the spectrum's layout (even, shifted x, shifted y)
-    st = g.yasym ? launch_col_convolve<T, 2>(ctx, g, B, spec, twz, nf, s)
+    // the z pass for the spectrum's layout (even, shifted x, shifted y, shifted z)
+    st = g.zasym ? launch_col_convolve<T, 3>(ctx, g, B, spec, twz, nf, s)
+       : g.yasym ? launch_col_convolve<T, 2>(ctx, g, B, spec, twz, nf, s)
        : g.xasym ? launch_col_convolve<T, 1>(ctx, g, B, spec, twz, nf, s)
                  : launch_col_convolve<T, 0>(ctx, g, B, spec, twz, nf, s);
     if (st != LGF_OK) return st;
@@ -504,7 +520,8 @@ lgf_status poisson_spectrum(lgf_ctx *ctx, const PoissonGeom &pg, double alpha, S
     if (Spectrum *hit = ctx->spectra.find(
             [&](const Spectrum &q) {
                 return q.M == shape && q.alpha == alpha && q.xasym == pg.xasym && q.xc == pg.xc && q.xP == pg.xP &&
-                       q.yasym == pg.yasym && q.yc == pg.yc && q.yP == pg.yP;
+                       q.yasym == pg.yasym && q.yc == pg.yc && q.yP == pg.yP && q.zasym == pg.zasym && q.zc == pg.zc &&
+                       q.zP == pg.zP;
             },
             ctx->counters.epoch)) {
         *out = hit;
@@ -538,8 +555,9 @@ lgf_status poisson_spectrum(lgf_ctx *ctx, const PoissonGeom &pg, double alpha, S
     // layouts: even x and y: reals [kz][ky <= My/2][kx]; shifted x: complex,
     // same shape; shifted y: complex [kz][ky < My][kx] (no symmetry in ky)
     const int nky = pg.yasym ? M[1] : M[1] / 2 + 1;
-    const bool cplx = pg.xasym || pg.yasym;
-    const size_t spec_elems = (size_t)pg.ld * nky * (M[2] / 2 + 1) * (cplx ? 2 : 1);
+    const int nkz = pg.zasym ? M[2] : M[2] / 2 + 1;   // and in kz where z is shifted
+    const bool cplx = pg.xasym || pg.yasym || pg.zasym;
+    const size_t spec_elems = (size_t)pg.ld * nky * nkz * (cplx ? 2 : 1);
     const size_t esz = ctx->prec == LGF_F64 ? 8 : 4;
     auto cleanup = [&]() {
         cudaFree(box);
@@ -553,15 +571,15 @@ lgf_status poisson_spectrum(lgf_ctx *ctx, const PoissonGeom &pg, double alpha, S
         cudaFree(spec);
         return fail(ctx, LGF_ENOMEM, "poisson: kernel spectrum scratch allocation failed");
     }
-    lgf_status st = kernel_window(ctx, table, M, pg.xc, pg.xP, pg.yc, pg.yP, box, s);
+    lgf_status st = kernel_window(ctx, table, pg, box, s);
     if (st == LGF_OK)
         st = run_passes<double>(ctx, g, box, nullptr, A, B, nullptr, 1, M[0], true, s);
     if (st == LGF_OK) {
         if (cplx) {
             if (esz == 8)
-                k_extract_c<double><<<152 * 4, 256, 0, s>>>(B, (Cx<double> *)spec, M[0], M[1], M[2], nky, pg.ld);
+                k_extract_c<double><<<152 * 4, 256, 0, s>>>(B, (Cx<double> *)spec, M[0], M[1], M[2], nky, nkz, pg.ld);
             else
-                k_extract_c<float><<<152 * 4, 256, 0, s>>>(B, (Cx<float> *)spec, M[0], M[1], M[2], nky, pg.ld);
+                k_extract_c<float><<<152 * 4, 256, 0, s>>>(B, (Cx<float> *)spec, M[0], M[1], M[2], nky, nkz, pg.ld);
         } else if (esz == 8) {
             k_extract<double><<<152 * 4, 256, 0, s>>>(B, (double *)spec, M[0], M[1], M[2], pg.ld);
         } else {
@@ -585,6 +603,9 @@ lgf_status poisson_spectrum(lgf_ctx *ctx, const PoissonGeom &pg, double alpha, S
     sp->yasym = pg.yasym;
     sp->yc = pg.yc;
     sp->yP = pg.yP;
+    sp->zasym = pg.zasym;
+    sp->zc = pg.zc;
+    sp->zP = pg.zP;
     sp->dev = spec;
     *out = ctx->spectra.insert(std::move(sp), ctx->counters.epoch, [&] { before_evict(ctx); },
                                &ctx->counters.plans_evicted);
@@ -748,7 +769,8 @@ lgf_status run_ragged(lgf_ctx *ctx, const RagPart *parts, int n, cudaStream_t s,
         z.t0 = g.t0[2];
         z.nt = g.Lt[2];
         z.nf = q.nf;
-        const int spec = g.yasym ? 2 : g.xasym ? 1 : 0;
+        z.ysym = !g.yasym;
+        const int spec = g.zasym ? 3 : g.yasym ? 2 : g.xasym ? 1 : 0;
         zc.add({g.M[2], spec, sizeof(T) == 4 ? g.zvar : 0}, z);
         if constexpr (sizeof(T) == 4) {   // the fused y+x inverse where it applies
             int rpb = 0;
@@ -795,7 +817,8 @@ lgf_status run_ragged(lgf_ctx *ctx, const RagPart *parts, int n, cudaStream_t s,
              const auto &key = zc.keys[k];
              pk::ConvJob<T> *j = zc.jobs[k].data();
              const int nj = (int)zc.jobs[k].size();
-             return key[1] == 2   ? launch_col_convolve_rag<T, 2>(ctx, key[0], key[2], j, nj, bs)
+             return key[1] == 3   ? launch_col_convolve_rag<T, 3>(ctx, key[0], key[2], j, nj, bs)
+                    : key[1] == 2 ? launch_col_convolve_rag<T, 2>(ctx, key[0], key[2], j, nj, bs)
                     : key[1] == 1 ? launch_col_convolve_rag<T, 1>(ctx, key[0], key[2], j, nj, bs)
                                   : launch_col_convolve_rag<T, 0>(ctx, key[0], key[2], j, nj, bs);
          })) != LGF_OK)

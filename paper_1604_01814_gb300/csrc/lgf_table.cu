@@ -222,8 +222,8 @@ __global__ void k_lookup(const double *table, int R, const int32_t *off, int64_t
 // Circular embedding of G_L on an Mx x My x Mz box: even along z
 // (h[m] = G_L(min(m, M - m))); along x and y the window h[m] = G_L(m + c) for
 // m < P and G_L(m - M + c) above (c = 0, P = M/2 is the even one).
-__global__ void k_window(const double *table, int R, int Mx, int My, int Mz, int xc, int xP, int yc, int yP,
-                         double *box)
+__global__ void k_window(const double *table, int R, int Mx, int My, int Mz, int xc, int xP, int yc, int yP, int zc,
+                         int zP, double *box)
 {
     const int64_t n = (int64_t)Mx * My * Mz;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
@@ -232,7 +232,8 @@ __global__ void k_window(const double *table, int R, int Mx, int My, int Mz, int
         const int z = (int)(i / ((int64_t)Mx * My));
         const int dxo = x < xP ? x + xc : x - Mx + xc;
         const int dyo = y < yP ? y + yc : y - My + yc;
-        box[i] = lgf_value(table, R, abs(dxo), abs(dyo), min(z, Mz - z));
+        const int dzo = z < zP ? z + zc : z - Mz + zc;
+        box[i] = lgf_value(table, R, abs(dxo), abs(dyo), abs(dzo));
     }
 }
 
@@ -562,10 +563,10 @@ lgf_status direct_samples(lgf_ctx *ctx, const lgf_blockset *src, const void *f_f
     return e == cudaSuccess ? LGF_OK : cuda_fail(ctx, e, "error estimate: direct samples");
 }
 
-lgf_status kernel_window(lgf_ctx *ctx, const double *table, const int M[3], int xc, int xP, int yc, int yP,
-                         double *box, cudaStream_t s)
+lgf_status kernel_window(lgf_ctx *ctx, const double *table, const PoissonGeom &g, double *box, cudaStream_t s)
 {
-    k_window<<<152 * 8, 256, 0, s>>>(table, ctx->table_radius, M[0], M[1], M[2], xc, xP, yc, yP, box);
+    k_window<<<152 * 8, 256, 0, s>>>(table, ctx->table_radius, g.M[0], g.M[1], g.M[2], g.xc, g.xP, g.yc, g.yP, g.zc,
+                                     g.zP, box);
     LGF_CHECK_LAUNCH(ctx, "window kernel");
     return LGF_OK;
 }

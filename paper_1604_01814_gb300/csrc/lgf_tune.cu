@@ -145,7 +145,7 @@ lgf_status tune_poisson(lgf_ctx *ctx, PoissonPlan *pl, int nf, double kalpha, cu
         if (before.count(&q)) return false;
         const bool winner = q.M == std::array<int, 3>{gw.M[0], gw.M[1], gw.M[2]} && q.alpha == kalpha &&
                             q.xasym == gw.xasym && q.xc == gw.xc && q.xP == gw.xP && q.yasym == gw.yasym &&
-                            q.yc == gw.yc && q.yP == gw.yP;
+                            q.yc == gw.yc && q.yP == gw.yP && q.zasym == gw.zasym && q.zc == gw.zc && q.zP == gw.zP;
         return !winner;
     });
     if (timed) {

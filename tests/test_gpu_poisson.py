@@ -277,3 +277,37 @@ def test_every_transform_length(M, axis, prec, ctx64, ctx32, oracle):
     f = np.random.default_rng(M + axis).uniform(-1, 1, (1, 1, c.shape[0], b ** 3))
     p = li.Problem("line", b, c, c.copy(), f)
     assert rel_linf(run_poisson(ctx, p), oracle_fields(oracle, p)) < TOL[prec]
+
+
+@pytest.mark.parametrize("prec", ["f64", "f32"])
+@pytest.mark.parametrize("b,src,sat,tgt", [(8, (1, 1, 1), (2, 1, 1), (6, 3, 5)),     # all three axes shifted
+                                           (8, (1, 3, 1), (0, 0, 4), (6, 3, 5)),     # y even
+                                           (8, (3, 1, 1), (0, 0, 0), (3, 6, 5)),     # x even
+                                           (8, (1, 1, 2), (9, -3, 7), (5, 4, 5)),    # sources past the targets
+                                           (8, (2, 1, 1), (-4, 2, -9), (6, 3, 10)),  # and before them
+                                           (16, (1, 1, 4), (1, 0, 2), (5, 2, 8)),    # 192 points along z
+                                           (16, (1, 1, 2), (1, 0, 2), (5, 2, 17)),   # 320
+                                           (32, (1, 1, 4), (0, 0, 1), (4, 1, 8)),    # 384
+                                           (32, (1, 1, 2), (0, 0, 1), (3, 1, 5))])   # 256
+def test_shifted_z_window(prec, b, src, sat, tgt, ctx64, ctx32, oracle):
+    """Targets that outreach the sources along z (and along x or y, which the
+    shift of z follows): sampled targets against the oracle, and a batch of the
+    problem and its mirror in z equal to the single applies bit for bit."""
+    import paper_1604_01814_gb300 as lgf
+    ctx = ctx64 if prec == "f64" else ctx32
+    rng = np.random.default_rng(b + sum(tgt))
+    t, probs = li.box_blocks(*tgt), []
+    for origin in (sat, (sat[0], sat[1], tgt[2] - src[2] - sat[2])):
+        sb = li.box_blocks(*src, origin=origin)
+        probs.append(li.Problem("z", b, sb, t, rng.uniform(-1, 1, (1, 2, sb.shape[0], b ** 3))))
+    single = [run_poisson(ctx, p, dx=0.5) for p in probs]
+    idx = rng.choice(t.shape[0] * b ** 3, size=600, replace=False)
+    for p, got in zip(probs, single):
+        assert rel_linf(got[:, :, idx], oracle_fields(oracle, p, idx, dx=0.5)) < TOL[prec]
+    batch = [dict(b=b, src=p.src, tgt=p.tgt, f=torch.tensor(p.f.reshape(-1), dtype=ctx.dtype, device="cuda"),
+                  u=torch.empty(2 * t.shape[0] * b ** 3, dtype=ctx.dtype, device="cuda"), ncomp=2, dx=0.5,
+                  op=lgf.LGF_OP_POISSON) for p in probs]
+    ctx.batch_apply(batch)
+    torch.cuda.synchronize()
+    for q, got in zip(batch, single):
+        assert np.array_equal(q["u"].cpu().numpy().astype(np.float64).reshape(got.shape), got)
