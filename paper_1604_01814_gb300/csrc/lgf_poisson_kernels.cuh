@@ -435,16 +435,17 @@ __global__ void __launch_bounds__(W * Plan<ML>::TPC) k_col_inverse(const Cx<T> *
 // for big boxes the spectrum is larger than L2.  Source and target planes
 // lie in [0, M/2): the first stage skips its zero upper inputs and the last
 // stage forms only its lower outputs.
-// Resident CTAs per SM that the register allocation must allow (FP32 at the
-// lengths 256 (32 warps), 320, 384 and 512 (24 warps) and the long mixed
-// lengths (2 CTAs); no spills).
+// Resident CTAs per SM that the register allocation must allow (FP32): four of
+// 256 threads up to length 256 (64 registers; the 64-plate batch 3.88 -> 3.82 ms against
+// the compiler's own choice below 160), five of 160 at 320, three at 384 and 512, two
+// at the long mixed lengths (no spills beyond a few bytes).
 // ZV = 1 (the tuner's alternative, FP32 only) asks for one more resident CTA
 // per SM than the default, i.e. a tighter register cap (where the default
-// leaves the choice to the compiler: 4 up to length 192, 3 above).
+// leaves the choice to the compiler, 3).
 template <typename T, int ML, int ZV = 0>
 struct ConvOcc {
-    static constexpr int base = sizeof(T) == 4 ? (ML == 160 || ML == 192 || ML == 256 ? 4 : ML == 320 ? 5 : ML == 384 || ML == 512 ? 3 : ML == 640 || ML == 1536 || ML == 2560 || ML == 3072 ? 2 : 1) : 1;
-    static constexpr int value = ZV == 0 ? base : (base == 1 ? (ML <= 192 ? 4 : 3) : base + 1);
+    static constexpr int base = sizeof(T) == 4 ? (ML <= 256 ? 4 : ML == 320 ? 5 : ML == 384 || ML == 512 ? 3 : ML == 640 || ML == 1536 || ML == 2560 || ML == 3072 ? 2 : 1) : 1;
+    static constexpr int value = ZV == 0 ? base : (base == 1 ? 3 : base + 1);
 };
 
 // SPEC: 0 the real spectrum of the even embedding ([kz][ky <= My/2][kx]);
