@@ -145,16 +145,25 @@ def load(path: str = LIB_PATH):
     return L
 
 
+_COORDS = lgf_blockset.coords.offset
+
+
 def _blockset(b: int, coords) -> tuple:
-    c = np.ascontiguousarray(np.asarray(coords, dtype=np.int32).reshape(-1, 3))
-    bs = lgf_blockset(int(b), int(c.shape[0]), c.ctypes.data_as(ctypes.POINTER(ctypes.c_int32)))
+    # (an [n][3] int32 array is taken as it is, and the pointer is stored through the
+    # struct's memory: the conversions and data_as cost 4 us a set, more than two
+    # kernel launches)
+    c = coords
+    if not (type(c) is np.ndarray and c.dtype == np.int32 and c.ndim == 2 and c.shape[1] == 3 and c.flags.c_contiguous):
+        c = np.ascontiguousarray(np.asarray(coords, dtype=np.int32).reshape(-1, 3))
+    bs = lgf_blockset(int(b), c.shape[0])
+    ctypes.c_void_p.from_buffer(bs, _COORDS).value = c.ctypes.data
     return bs, c   # keep the array alive with the struct
 
 
 def _stream_ptr(stream) -> Optional[int]:
     if stream is None:
         import torch
-        return torch.cuda.current_stream().cuda_stream or None
+        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device()) or None
     if isinstance(stream, int):
         return stream or None
     return stream.cuda_stream or None

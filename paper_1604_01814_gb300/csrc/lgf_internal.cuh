@@ -162,6 +162,14 @@ struct CurlPlan {
     uint64_t used = 0;
     ~CurlPlan();
 };
+// A block set with its grown set, the targets of the Poisson problem behind a
+// staggered operator (dir +1: and the +x, +y, +z neighbours, for the refresh;
+// -1: and the -x, -y, -z ones, for the stage).  Host data only.
+struct GrownSet {
+    int dir = 0;
+    std::vector<int32_t> coords, grown;
+    uint64_t used = 0;
+};
 constexpr int kBranches = 8;        // most concurrent branches of a batch
 constexpr int kDefaultBranches = 4; // branches of an untuned batch
 
@@ -195,6 +203,7 @@ struct lgf_ctx {
     std::vector<std::unique_ptr<lgf::IntfWeights>> weights;
     lgf::LruCache<lgf::CurlPlan> cplans{64};
     lgf::LruCache<lgf::IBPlan> ibplans{64};
+    lgf::LruCache<lgf::GrownSet> grown{64};
     lgf::CacheCounters counters;
 
     // grow-only scratch, one set per concurrent branch of lgf_batch_apply

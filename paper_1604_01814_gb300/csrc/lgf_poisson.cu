@@ -417,13 +417,17 @@ const void *twiddles(lgf_ctx *ctx, int M, bool dbl, lgf_status *st)
 lgf_status poisson_plan(lgf_ctx *ctx, const lgf_blockset *src, const lgf_blockset *tgt, PoissonPlan **out)
 {
     const int b = src->b;
-    const std::vector<int32_t> sv(src->coords, src->coords + 3 * (size_t)src->nblocks);
-    const std::vector<int32_t> tv(tgt->coords, tgt->coords + 3 * (size_t)tgt->nblocks);
+    auto same = [](const std::vector<int32_t> &v, const lgf_blockset *bs) {
+        return v.size() == 3 * (size_t)bs->nblocks && std::equal(v.begin(), v.end(), bs->coords);
+    };
     if (PoissonPlan *hit = ctx->pplans.find(
-            [&](const PoissonPlan &p) { return p.b == b && p.src == sv && p.tgt == tv; }, ctx->counters.epoch)) {
+            [&](const PoissonPlan &p) { return p.b == b && same(p.src, src) && same(p.tgt, tgt); },
+            ctx->counters.epoch)) {
         *out = hit;
         return LGF_OK;
     }
+    const std::vector<int32_t> sv(src->coords, src->coords + 3 * (size_t)src->nblocks);
+    const std::vector<int32_t> tv(tgt->coords, tgt->coords + 3 * (size_t)tgt->nblocks);
     int slo[3], shi[3], tlo[3], thi[3], lo[3], hi[3];
     for (int d = 0; d < 3; ++d) {
         slo[d] = tlo[d] = INT32_MAX;
