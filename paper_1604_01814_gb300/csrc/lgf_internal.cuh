@@ -245,6 +245,9 @@ struct lgf_ctx {
 
     // optional per-kernel timing with CUDA events on the launch stream
     bool prof = false;
+    // the next pass launches follow their predecessor on the stream directly (set
+    // around the passes of a single apply: no event between them, no capture)
+    bool chain = false;
     struct ProfRec {
         int name;
         cudaEvent_t a, b;

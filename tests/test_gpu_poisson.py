@@ -311,3 +311,34 @@ def test_shifted_z_window(prec, b, src, sat, tgt, ctx64, ctx32, oracle):
     torch.cuda.synchronize()
     for q, got in zip(batch, single):
         assert np.array_equal(q["u"].cpu().numpy().astype(np.float64).reshape(got.shape), got)
+
+
+@pytest.mark.parametrize("b,extent,nf", [(8, (3, 3, 3), 1), (16, (4, 3, 3), 3), (32, (4, 4, 4), 1), (32, (5, 4, 4), 3)])
+def test_chained_passes_repeated_and_captured(b, extent, nf, ctx32, oracle):
+    """The passes of a single apply overlap their launches on small grids (up
+    to a few waves) and follow one another plainly on large ones and inside a
+    capture: back to back applies that reuse the scratch, the profiled passes
+    (events between them) and a captured apply give the same bits."""
+    c = li.box_blocks(*extent)
+    f = [torch.randn(nf * c.shape[0] * b ** 3, device="cuda", generator=torch.Generator("cuda").manual_seed(k))
+         for k in range(3)]
+    u = [torch.full_like(v, float("nan")) for v in f]
+    for _ in range(20):
+        for a, v in zip(f, u):
+            ctx32.poisson_apply(b, c, c, a, v, ncomp=nf)
+    ref = [torch.full_like(v, float("nan")) for v in f]
+    ctx32.profile_enable(True)
+    for a, v in zip(f, ref):
+        ctx32.poisson_apply(b, c, c, a, v, ncomp=nf)
+    torch.cuda.synchronize()
+    ctx32.profile_enable(False)
+    cap = torch.full_like(f[0], float("nan"))
+    s, g = torch.cuda.Stream(), torch.cuda.CUDAGraph()
+    s.wait_stream(torch.cuda.current_stream())
+    with torch.cuda.graph(g, stream=s):
+        ctx32.poisson_apply(b, c, c, f[0], cap, ncomp=nf)
+    g.replay()
+    torch.cuda.synchronize()
+    for a, v in zip(u, ref):
+        assert torch.equal(a, v)
+    assert torch.equal(cap, ref[0])
