@@ -349,8 +349,7 @@ struct Col8<double> {
 // fetched (16 + 2 RMAX) / 16 times, from L2 or L1.  Staging slabs in shared memory with 4
 // outputs per thread read it (4 + 2 RMAX) / 4 times from there: the l1tex pipe was
 // 70 % busy and 556 blocks of 16^3 (3 fields, RMAX 8) took 16.2 us, now 12.3; the
-// 64-plate batch's launch 281, now 215.  Blocks of 8 keep the staged pass: a plane has
-// too few columns for a CTA.
+// 64-plate batch's launch 281, now 215.
 // The order of the additions is that of k_sep_win.
 template <typename T, int LB>
 struct ZCfg {
@@ -359,6 +358,14 @@ struct ZCfg {
     static constexpr int THREADS = LANES < 128 ? LANES : 128;
     static constexpr int NY = (LANES / THREADS) * (b / V);   // grid.y: slices of the plane, runs along z
 };
+// Whether a launch over `blocks` output blocks (times jobs and fields) takes k_sep_z or
+// the staged k_sep_win.  Measured in FP32, staged over k_sep_z time: blocks of 16,
+// 1.03 to 1.6 from 8 to 3000 blocks and at every window; blocks of 32 (two runs along
+// z, so more of the window is fetched twice), window up to 8: 0.9 to 1.0 up to 125
+// blocks, 1.04 at 192, 1.15 at 375; windows 12 and 16: 0.75 to 1.02.  Equal in FP64, which
+// its arithmetic bounds.  Blocks of 8: a plane has too few columns for a CTA.
+template <int LB, int RMAX>
+constexpr bool z_march(int64_t blocks) { return LB == 4 || (LB == 5 && RMAX <= 8 && blocks >= 192); }
 template <typename T, int LB, int RMAX, class Tab = SepJobs<T>>
 __global__ void __launch_bounds__(ZCfg<T, LB>::THREADS)
     k_sep_z(const __grid_constant__ Tab jobs, const int *__restrict__ nbr_arg, int nr_arg)
@@ -714,16 +721,18 @@ lgf_status launch_m(lgf_ctx *ctx, int nout, const SepJobs<T> &jobs, cudaStream_t
     }
     if constexpr (AX == 2 && LB >= 4) {
         using Z = ZCfg<T, LB>;
-        k_sep_z<T, LB, RMAX><<<dim3(nout, Z::NY, jobs.n * jobs.nf), Z::THREADS, 0, s>>>(jobs, nbr, nr);
-    } else {
-        auto kern = k_sep_win<T, LB, AX, RMAX>;
-        if (smem > 48 * 1024) {
-            cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-            if (e != cudaSuccess) return cuda_fail(ctx, e, "cudaFuncSetAttribute");
+        if (z_march<LB, RMAX>((int64_t)nout * jobs.n * jobs.nf)) {
+            k_sep_z<T, LB, RMAX><<<dim3(nout, Z::NY, jobs.n * jobs.nf), Z::THREADS, 0, s>>>(jobs, nbr, nr);
+            return LGF_OK;
         }
-        dim3 grid(nout, b / C::NS, jobs.n * jobs.nf);
-        kern<<<grid, C::THREADS, smem, s>>>(jobs, nbr, nr);
     }
+    auto kern = k_sep_win<T, LB, AX, RMAX>;
+    if (smem > 48 * 1024) {
+        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return cuda_fail(ctx, e, "cudaFuncSetAttribute");
+    }
+    dim3 grid(nout, b / C::NS, jobs.n * jobs.nf);
+    kern<<<grid, C::THREADS, smem, s>>>(jobs, nbr, nr);
     return LGF_OK;
 }
 
@@ -771,22 +780,24 @@ lgf_status launch_z_rag_m(lgf_ctx *ctx, SepRagJob<T> *jobs, int n, cudaStream_t 
 {
     if constexpr (LB >= 4) {
         using Z = ZCfg<T, LB>;
-        return rag_send_sep<T>(ctx, jobs, n, [&](unsigned gx, const SepRag<T> &t) {
-            k_sep_z<T, LB, RMAX, SepRag<T>><<<dim3(gx, Z::NY, 1), Z::THREADS, 0, s>>>(t, nullptr, 0);
-        });
-    } else {
-        using C = Cfg<T, LB, 2>;
-        constexpr int b = 1 << LB, E = b + 2 * RMAX;
-        constexpr size_t smem = sizeof(T) * (size_t)C::NS * b * E;
-        auto kern = k_sep_win<T, LB, 2, RMAX, SepRag<T>>;
-        if (smem > 48 * 1024) {
-            cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-            if (e != cudaSuccess) return cuda_fail(ctx, e, "cudaFuncSetAttribute");
-        }
-        return rag_send_sep<T>(ctx, jobs, n, [&](unsigned gx, const SepRag<T> &t) {
-            kern<<<dim3(gx, b / C::NS, 1), C::THREADS, smem, s>>>(t, nullptr, 0);
-        });
+        int64_t blocks = 0;
+        for (int i = 0; i < n; ++i) blocks += (int64_t)jobs[i].nitems * jobs[i].nf;
+        if (z_march<LB, RMAX>(blocks))
+            return rag_send_sep<T>(ctx, jobs, n, [&](unsigned gx, const SepRag<T> &t) {
+                k_sep_z<T, LB, RMAX, SepRag<T>><<<dim3(gx, Z::NY, 1), Z::THREADS, 0, s>>>(t, nullptr, 0);
+            });
     }
+    using C = Cfg<T, LB, 2>;
+    constexpr int b = 1 << LB, E = b + 2 * RMAX;
+    constexpr size_t smem = sizeof(T) * (size_t)C::NS * b * E;
+    auto kern = k_sep_win<T, LB, 2, RMAX, SepRag<T>>;
+    if (smem > 48 * 1024) {
+        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return cuda_fail(ctx, e, "cudaFuncSetAttribute");
+    }
+    return rag_send_sep<T>(ctx, jobs, n, [&](unsigned gx, const SepRag<T> &t) {
+        kern<<<dim3(gx, b / C::NS, 1), C::THREADS, smem, s>>>(t, nullptr, 0);
+    });
 }
 
 template <typename T, int LB, int AX>

@@ -141,3 +141,19 @@ def test_every_window_class_more_block_shapes(ctx32, ctx64, oracle, prec, b, see
         ref = oracle_intf(oracle, p, alpha)
         if np.abs(ref).max() > 0:
             assert rel_linf(run_intf(ctx, p, alpha), ref) < TOL[prec], alpha
+
+
+@pytest.mark.parametrize("prec", ["f32", "f64"])
+@pytest.mark.parametrize("nf", [1, 2])
+def test_z_pass_rule_on_blocks_of_32(ctx32, ctx64, prec, nf):
+    """Blocks of 32 take one z pass below 192 blocks and fields and another
+    from there on: the fields of one call equal the calls of one field each bit
+    for bit on both sides of the line (100 and 200)."""
+    ctx = ctx64 if prec == "f64" else ctx32
+    b, c = 32, li.box_blocks(5, 5, 4)
+    f = torch.randn(nf, c.shape[0] * b ** 3, dtype=ctx.dtype, device="cuda")
+    u, one = torch.full_like(f, float("nan")), torch.full_like(f, float("nan"))
+    ctx.intfactor_apply(0.02, b, c, c, f, u, ncomp=nf)
+    for k in range(nf):
+        ctx.intfactor_apply(0.02, b, c, c, f[k], one[k])
+    assert torch.equal(u, one)
