@@ -450,7 +450,8 @@ LGF_API lgf_status lgf_wait_selftest(lgf_ctx *ctx, int64_t cycles, void *stream)
 /* Autotuner.  A Poisson plan's geometry has free choices that the method
    leaves open (Sec. 2.2 fixes only the convolution): the embedding of x and
    of y (the even circular embedding of G_L, M >= 2L - 1 on the union extent
-   L, or the shifted window, M >= Ls + Lt - 1), the transform length along
+   L, or the shifted window, M >= Ls + Lt - 1; z takes the window where x or
+   y does and it is shorter), the transform length along
    each axis (the smallest supported length, or the next one, whose radix
    plan may run faster) and the register cap of the z pass (FP32); a batch
    also has its branch count (1, 2, 4 or 8 concurrent streams).  With tuning on,

@@ -9,9 +9,10 @@
 // register (the distance d is a compile-time constant after unrolling).
 // Shared-memory traffic per output is (V + 2 RMAX) / V values instead of
 // 2R + 1.  In FP32 the accumulators go in pairs through the packed FP32x2 FMA
-// (two lane-wise fma.rn per instruction, the scalar loop's bits): adjacent x
-// values in the y and z passes, adjacent y rows in the x pass of the fused
-// x+y kernel.
+// (two lane-wise fma.rn per instruction, the scalar loop's bits) for adjacent x
+// values in the y and z passes.  This is the form of the single-axis passes; the
+// fused x+y pass and the z pass of larger blocks below make 8 or 16 outputs per
+// thread.
 #pragma once
 #include <algorithm>
 #include <type_traits>
