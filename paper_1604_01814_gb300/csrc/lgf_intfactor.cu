@@ -508,7 +508,10 @@ static lgf_status run_sep_jobs(lgf_ctx *ctx, IntfPlan *pl, const IntfJob *jobs, 
             LGF_CHECK_LAUNCH(ctx, "intfactor xy pass");
             prof_end(ctx, s, ph);
             const int pz = prof_begin(ctx, s, "intfactor_pass_z");
-            st = launch_sep_window<T>(ctx, 2, b, ntgt, jz, s, pl->pass[2].nbr_dev, nr, &done);
+            {
+                const ChainScope chain(ctx, s);   // the z pass directly follows the x+y pass
+                st = launch_sep_window<T>(ctx, 2, b, ntgt, jz, s, pl->pass[2].nbr_dev, nr, &done);
+            }
             if (st != LGF_OK) return st;
             if (!done) return fail(ctx, LGF_ECUDA, "intfactor: z window pass unavailable after the xy pass");
             LGF_CHECK_LAUNCH(ctx, "intfactor z pass");

@@ -221,6 +221,7 @@ __global__ void __launch_bounds__(Cfg<T, LB, AX>::THREADS)
     const T *inf = J.in + field * J.in_stride;
     T *outf = J.out + field * J.out_stride;
 
+    chain_wait();
     // ---- stage [slab + halo] with 16-byte loads ----
     constexpr int rowlen = AX == 0 ? E : b;
     constexpr int nrows = AX == 0 ? NS * b : NS * E;
@@ -393,9 +394,10 @@ __global__ void __launch_bounds__(ZCfg<T, LB>::THREADS)
         }
     };
     VT cur[CH], nxt[CH], acc[V];
-    load(cur, 0);
     WinW<T, RMAX> W;
     load_weights(W, J.w, J.R);
+    chain_wait();
+    load(cur, 0);
 #pragma unroll
     for (int v = 0; v < V; ++v) acc[v] = VT{};
 #pragma unroll
@@ -566,6 +568,7 @@ __global__ void __launch_bounds__(XYCfg<T, LB, RMAX>::THREADS)
     constexpr int b = C::b, bm = b - 1, NV = C::NV, NS = C::NS, HL = RMAX, LD = C::LD;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     T *s = reinterpret_cast<T *>(smem_raw);         // [NS][EY][LD], planes PL apart
+    chain_wait();
     __shared__ int nbs[(2 * kMaxWinNr + 2) * (2 * kMaxWinNr + 1)];
     const int o1 = at.items[2 * at.item], o2 = at.items[2 * at.item + 1];
     const bool pair = o2 >= 0;                      // uniform over the CTA
@@ -723,8 +726,9 @@ lgf_status launch_m(lgf_ctx *ctx, int nout, const SepJobs<T> &jobs, cudaStream_t
     if constexpr (AX == 2 && LB >= 4) {
         using Z = ZCfg<T, LB>;
         if (z_march<LB, RMAX>((int64_t)nout * jobs.n * jobs.nf)) {
-            k_sep_z<T, LB, RMAX><<<dim3(nout, Z::NY, jobs.n * jobs.nf), Z::THREADS, 0, s>>>(jobs, nbr, nr);
-            return LGF_OK;
+            const cudaError_t e = chain_launch(ctx && ctx->chain, k_sep_z<T, LB, RMAX>, dim3(nout, Z::NY, jobs.n * jobs.nf),
+                                               Z::THREADS, 0, s, jobs, nbr, nr);
+            return e == cudaSuccess ? LGF_OK : cuda_fail(ctx, e, "intfactor z pass");
         }
     }
     auto kern = k_sep_win<T, LB, AX, RMAX>;
@@ -733,8 +737,8 @@ lgf_status launch_m(lgf_ctx *ctx, int nout, const SepJobs<T> &jobs, cudaStream_t
         if (e != cudaSuccess) return cuda_fail(ctx, e, "cudaFuncSetAttribute");
     }
     dim3 grid(nout, b / C::NS, jobs.n * jobs.nf);
-    kern<<<grid, C::THREADS, smem, s>>>(jobs, nbr, nr);
-    return LGF_OK;
+    const cudaError_t e = chain_launch(ctx && ctx->chain, kern, grid, C::THREADS, smem, s, jobs, nbr, nr);
+    return e == cudaSuccess ? LGF_OK : cuda_fail(ctx, e, "intfactor pass");
 }
 
 // Ragged launches: every job field but cta0 set; sent in tables of

@@ -335,18 +335,7 @@ lgf_status run_passes(lgf_ctx *ctx, const PoissonGeom &g, const T *f, T *u, Cx<T
     const int ld = g.ld;
     const int64_t planeA = (int64_t)g.ldA_y * ld, planeB = (int64_t)My * ld;
     if ((st = launch_row_forward<T>(ctx, g, f, A, twx, nf, lb, dense_ld, s)) != LGF_OK) return st;
-    // from here each pass directly follows its predecessor (unless events go
-    // between them, or a capture records them: its graph keeps full dependencies)
-    struct Chain {
-        lgf_ctx *c;
-        ~Chain() { c->chain = false; }
-    } chain{ctx};
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(s, &cap) != cudaSuccess) {
-        cudaGetLastError();
-        cap = cudaStreamCaptureStatusActive;
-    }
-    ctx->chain = !ctx->prof && cap == cudaStreamCaptureStatusNone;
+    const ChainScope chain(ctx, s);   // from here each pass directly follows its predecessor
     const pk::RowFlags fsrc{spectrum_mode ? nullptr : g.srcrow, lb};
     if ((st = launch_col_forward<T>(ctx, My, K, g.Ls[2], nf, A, B, g.s0[1], g.Ls[1], ld, ld, planeA, planeB, g.Astride,
                                     g.Bstride, twy, fsrc, s,

@@ -183,13 +183,7 @@ struct ColAddrW {   // element m of column w: m * W + w
     __device__ __forceinline__ int operator()(int w, int m) const { return m * W + w; }
 };
 // The twiddles, which no pass writes, may be fetched while the previous pass still
-// runs; everything else waits for it (chain_wait: at once unless the launch allows the
-// overlap, see chain_launch).
-__device__ __forceinline__ void chain_wait()
-{
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-}
+// runs; everything else waits for it (chain_wait).
 template <typename T>
 __device__ __forceinline__ void load_twiddles(Cx<T> *tw, const Cx<T> *__restrict__ twg, int M)
 {
@@ -1113,32 +1107,6 @@ inline lgf_status set_smem(lgf_ctx *ctx, K kern, size_t smem)
         if (e != cudaSuccess) return cuda_fail(ctx, e, "cudaFuncSetAttribute");
     }
     return LGF_OK;
-}
-
-// Launch a pass of one problem.  follows: the previous launch of the stream is the
-// previous pass of the same problem, so this one may start while that drains
-// (programmatic stream serialisation; its CTAs wait in load_twiddles, every CTA
-// before it touches the pass's data, so each pass still sees all of the one before).
-// It hides the launch and the twiddle fetch of four passes: 24^3 apply 26.6 -> 22.7 us,
-// FP64 32^3 box 51.2 -> 41.0, K(alpha)^-1 of 32 blocks 50.2 -> 43.6, sphere Poisson apply
-// 147 -> 138, sphere stage 766 -> 742.  Only for grids of a few waves: waiting CTAs of a
-// larger one hold the slots that the previous pass needs (with no limit the refresh of
-// 556 blocks took 668 us instead of 600, the 512x256x256 wake 6.43 ms instead of 6.12).
-constexpr int64_t kChainCtas = 4000;
-template <class... P, class... A>
-cudaError_t chain_launch(bool follows, void (*kern)(P...), dim3 grid, int threads, size_t smem, cudaStream_t s, A... args)
-{
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = grid;
-    cfg.blockDim = dim3(threads);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = s;
-    cudaLaunchAttribute at;
-    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at.val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = &at;
-    cfg.numAttrs = follows && (int64_t)grid.x * grid.y <= kChainCtas ? 1 : 0;
-    return cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
 }
 
 template <typename T, int ML>

@@ -157,3 +157,35 @@ def test_z_pass_rule_on_blocks_of_32(ctx32, ctx64, prec, nf):
     for k in range(nf):
         ctx.intfactor_apply(0.02, b, c, c, f[k], one[k])
     assert torch.equal(u, one)
+
+
+@pytest.mark.parametrize("prec", ["f32", "f64"])
+@pytest.mark.parametrize("b,extent,nf", [(4, (3, 3, 3), 1), (16, (3, 3, 3), 3), (32, (3, 2, 2), 1), (16, (11, 11, 11), 4)])
+def test_chained_z_pass_repeated_and_captured(ctx32, ctx64, prec, b, extent, nf):
+    """The z pass overlaps the end of the x+y pass on small grids (the last
+    shape is beyond that limit) and follows it plainly inside a capture or with
+    profiling events between them: back to back applies that reuse the scratch,
+    the profiled ones and a captured one give the same bits."""
+    ctx = ctx64 if prec == "f64" else ctx32
+    c = li.box_blocks(*extent)
+    f = [torch.randn(nf * c.shape[0] * b ** 3, dtype=ctx.dtype, device="cuda",
+                     generator=torch.Generator("cuda").manual_seed(k)) for k in range(3)]
+    u, ref = ([torch.full_like(v, float("nan")) for v in f] for _ in range(2))
+    for _ in range(20):
+        for a, v in zip(f, u):
+            ctx.intfactor_apply(0.1, b, c, c, a, v, ncomp=nf)
+    ctx.profile_enable(True)
+    for a, v in zip(f, ref):
+        ctx.intfactor_apply(0.1, b, c, c, a, v, ncomp=nf)
+    torch.cuda.synchronize()
+    ctx.profile_enable(False)
+    cap = torch.full_like(f[0], float("nan"))
+    s, g = torch.cuda.Stream(), torch.cuda.CUDAGraph()
+    s.wait_stream(torch.cuda.current_stream())
+    with torch.cuda.graph(g, stream=s):
+        ctx.intfactor_apply(0.1, b, c, c, f[0], cap, ncomp=nf)
+    g.replay()
+    torch.cuda.synchronize()
+    for a, v in zip(u, ref):
+        assert torch.equal(a, v)
+    assert torch.equal(cap, ref[0])
