@@ -352,7 +352,9 @@ struct Col8<double> {
 // outputs per thread read it (4 + 2 RMAX) / 4 times from there: the l1tex pipe was
 // 70 % busy and 556 blocks of 16^3 (3 fields, RMAX 8) took 16.2 us, now 12.3; the
 // 64-plate batch's launch 281, now 215.
-// The order of the additions is that of k_sep_win.
+// The order of the additions is that of k_sep_win.  The field comes by ordinary loads:
+// a chained launch starts while the x+y pass still writes it, and the read-only path
+// (__ldg) is only for data that nobody writes during the kernel.
 template <typename T, int LB>
 struct ZCfg {
     static constexpr int b = 1 << LB, V = 16;
@@ -389,7 +391,7 @@ __global__ void __launch_bounds__(ZCfg<T, LB>::THREADS)
         for (int i = 0; i < CH; ++i) {
             const int e = z0 + c * CH + i - RMAX;
             const int bi = nb[e >> LB];
-            v[i] = bi >= 0 ? __ldg(reinterpret_cast<const VT *>(inf + ((int64_t)bi << (3 * LB)) + ((e & bm) << (2 * LB))))
+            v[i] = bi >= 0 ? *reinterpret_cast<const VT *>(inf + ((int64_t)bi << (3 * LB)) + ((e & bm) << (2 * LB)))
                            : VT{};
         }
     };

@@ -183,7 +183,13 @@ struct ColAddrW {   // element m of column w: m * W + w
     __device__ __forceinline__ int operator()(int w, int m) const { return m * W + w; }
 };
 // The twiddles, which no pass writes, may be fetched while the previous pass still
-// runs; everything else waits for it (chain_wait).
+// runs; everything else waits for it (chain_wait).  A, B, f and u, which the passes
+// hand on, are therefore plain pointers in every body and kernel that may be
+// chained: const with __restrict__, or __restrict__ alone, promises that nobody
+// else writes them while the kernel runs, and a load under that promise may use the
+// read-only path or move ahead of chain_wait, when the previous pass still writes.
+// (The f of the x forward pass is not handed on by a pass, and that kernel is
+// never chained.)
 template <typename T>
 __device__ __forceinline__ void load_twiddles(Cx<T> *tw, const Cx<T> *__restrict__ twg, int M)
 {
@@ -254,7 +260,7 @@ __device__ __forceinline__ bool column_of(int cta, int w, int K, int nplanes, in
 // kernels below run it at their own blockIdx, the ragged kernels at the
 // coordinates of a CTA inside one job of a job table.)
 template <typename T, int ML, int W, bool HALF>
-__device__ __forceinline__ void col_forward_body(int bx, int by, const Cx<T> *__restrict__ in, Cx<T> *__restrict__ out,
+__device__ __forceinline__ void col_forward_body(int bx, int by, const Cx<T> *in, Cx<T> *out,
                                                  int K, int nplanes, int lo, int n, int64_t rs, int64_t os,
                                                  int64_t in_plane, int64_t out_plane, int64_t in_field,
                                                  int64_t out_field, const Cx<T> *__restrict__ twg, RowFlags rf)
@@ -338,7 +344,7 @@ __device__ __forceinline__ void col_forward_body(int bx, int by, const Cx<T> *__
 }
 
 template <typename T, int ML, int W, bool HALF>
-__global__ void __launch_bounds__(W * Plan<ML>::TPC) k_col_forward(const Cx<T> *__restrict__ in, Cx<T> *__restrict__ out,
+__global__ void __launch_bounds__(W * Plan<ML>::TPC) k_col_forward(const Cx<T> *in, Cx<T> *out,
                                                                      int K, int nplanes, int lo, int n, int64_t rs,
                                                                      int64_t os, int64_t in_plane, int64_t out_plane,
                                                                      int64_t in_field, int64_t out_field,
@@ -354,7 +360,7 @@ __global__ void __launch_bounds__(W * Plan<ML>::TPC) k_col_forward(const Cx<T> *
 // last stage forms only the lower half of its outputs (otherwise, the
 // shifted y window with targets past M/2, all of them).
 template <typename T, int ML, int W, bool HALF_OUT>
-__device__ __forceinline__ void col_inverse_body(int bx, int by, const Cx<T> *__restrict__ in, Cx<T> *__restrict__ out,
+__device__ __forceinline__ void col_inverse_body(int bx, int by, const Cx<T> *in, Cx<T> *out,
                                                  int K, int nplanes, int lo, int n, int64_t rs, int64_t os,
                                                  int64_t in_plane, int64_t out_plane, int64_t in_field,
                                                  int64_t out_field, const Cx<T> *__restrict__ twg)
@@ -421,7 +427,7 @@ __device__ __forceinline__ void col_inverse_body(int bx, int by, const Cx<T> *__
 }
 
 template <typename T, int ML, int W, bool HALF_OUT>
-__global__ void __launch_bounds__(W * Plan<ML>::TPC) k_col_inverse(const Cx<T> *__restrict__ in, Cx<T> *__restrict__ out,
+__global__ void __launch_bounds__(W * Plan<ML>::TPC) k_col_inverse(const Cx<T> *in, Cx<T> *out,
                                                                      int K, int nplanes, int lo, int n, int64_t rs,
                                                                      int64_t os, int64_t in_plane, int64_t out_plane,
                                                                      int64_t in_field, int64_t out_field,
@@ -460,7 +466,7 @@ struct ConvOcc {
 // points instead of 256 along z of the sphere set, whose Poisson apply went from 152.0
 // to 145.9 us in FP32 and from 3.53 to 3.05 ms in FP64.
 template <typename T, int ML, int W, int SPEC>
-__device__ __forceinline__ void col_convolve_body(int bx, int nf, Cx<T> *__restrict__ B, const void *__restrict__ specv,
+__device__ __forceinline__ void col_convolve_body(int bx, int nf, Cx<T> *B, const void *__restrict__ specv,
                                                   int K, int ld, int lds, int My, int ysym, int s0, int ns, int t0,
                                                   int nt, int64_t field, const Cx<T> *__restrict__ twg)
 {
@@ -582,7 +588,7 @@ __device__ __forceinline__ void col_convolve_body(int bx, int nf, Cx<T> *__restr
 }
 
 template <typename T, int ML, int W, int SPEC, int ZV>
-__global__ void __launch_bounds__(W * Plan<ML>::TPC, ConvOcc<T, ML, ZV>::value) k_col_convolve(Cx<T> *__restrict__ B, const void *__restrict__ specv,
+__global__ void __launch_bounds__(W * Plan<ML>::TPC, ConvOcc<T, ML, ZV>::value) k_col_convolve(Cx<T> *B, const void *__restrict__ specv,
                                                                       int K, int ld, int lds, int My, int ysym, int s0,
                                                                       int ns, int t0, int nt, int64_t field,
                                                                       const Cx<T> *__restrict__ twg)
@@ -837,7 +843,7 @@ __global__ void __launch_bounds__(RowLay<T, ML>::THREADS, RowLay<T, ML>::OCC)
 // lower half of the last stage's outputs is formed; otherwise (the shifted x
 // window, targets up to M) every output is.
 template <typename T, int ML, bool HALF_OUT>
-__device__ __forceinline__ void row_inverse_body(int bx, int by, const Cx<T> *__restrict__ A, T *__restrict__ u,
+__device__ __forceinline__ void row_inverse_body(int bx, int by, const Cx<T> *A, T *u,
                                                  const PoissonGeom &g, const Cx<T> *__restrict__ twg, int npairs,
                                                  int lb)
 {
@@ -890,7 +896,7 @@ __device__ __forceinline__ void row_inverse_body(int bx, int by, const Cx<T> *__
     if (!live) return;
     const T sc = T(g.scale);
     const int bm = g.b - 1;
-    const int *mrow = g.tgtmap + ((zi >> lb) * g.nbt[1] + (yi >> lb)) * g.nbt[0];
+    const int *__restrict__ mrow = g.tgtmap + ((zi >> lb) * g.nbt[1] + (yi >> lb)) * g.nbt[0];
     const int inner = (((zi & bm) << lb) + (yi & bm)) << lb;
     T *uu = u + by * g.ustride;
     constexpr int R0 = P::R0;
@@ -919,7 +925,7 @@ __device__ __forceinline__ void row_inverse_body(int bx, int by, const Cx<T> *__
 
 template <typename T, int ML, bool HALF_OUT>
 __global__ void __launch_bounds__(RowLay<T, ML>::THREADS, RowLay<T, ML>::OCC)
-    k_row_inverse(const Cx<T> *__restrict__ A, T *__restrict__ u, PoissonGeom g, const Cx<T> *__restrict__ twg,
+    k_row_inverse(const Cx<T> *A, T *u, PoissonGeom g, const Cx<T> *__restrict__ twg,
                   int npairs, int lb)
 {
     row_inverse_body<T, ML, HALF_OUT>(blockIdx.x, blockIdx.y, A, u, g, twg, npairs, lb);
