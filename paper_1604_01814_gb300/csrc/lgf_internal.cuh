@@ -262,17 +262,18 @@ struct lgf_ctx {
 namespace lgf {
 
 // Launch a pass of one problem.  follows: the previous launch of the stream is the
-// previous pass of the same problem, so this one may start while that drains
+// previous pass of the same problem, so this one may be set up while that drains
 // (programmatic stream serialisation).  Every thread calls chain_wait before it
 // touches the pass's data, so each pass still sees all of the one before; what no pass
-// writes (twiddles, weights, neighbour tables) may be read ahead of it.  It hides
-// the launch and those fetches: 24^3 apply 26.6 -> 22.7 us, FP64 32^3 box 51.2 -> 41.0,
-// K(alpha)^-1 of 32 blocks 50.2 -> 43.6, sphere Poisson apply 147 -> 138, sphere stage 766 ->
-// 742, and with the integrating factor's z pass, sphere E(alpha) 36.9 -> 34.8, stage 737.
-// Only for grids of a few waves: waiting CTAs of a larger one hold the slots that
-// the previous pass needs (with no limit the refresh of 556 blocks took 668 us instead of
-// 600, the 512x256x256 wake 6.43 ms instead of 6.12).
-constexpr int64_t kChainCtas = 4000;
+// writes (twiddles, weights, neighbour tables) may be read ahead of it.
+// No pass releases its dependents early (griddepcontrol.launch_dependents): their CTAs
+// start when the last CTA of the predecessor has exited, on empty SMs.  Released at
+// entry, they were placed while the predecessor ran, all on the SMs that it had left
+// free, and stayed there: E(0.75) of 8 FP64 blocks of 32 took 171 us (76 unchained, 74
+// now), the FP64 box of 96x32x32 275 us (190, 179), 16x128x128 in FP32 57 (40, 31),
+// 32x32x384 56 (44, 33).  Against plain launches it hides the launch and those fetches:
+// 24^3 apply 26.6 -> 20.2 us, sphere Poisson apply 147 -> 138, sphere stage 766 -> 742; over
+// 1000 calls from 16^3 to 10^8 points none is slower, so there is no limit on the grid.
 template <class... P, class... A>
 cudaError_t chain_launch(bool follows, void (*kern)(P...), dim3 grid, int threads, size_t smem, cudaStream_t s, A... args)
 {
@@ -285,14 +286,10 @@ cudaError_t chain_launch(bool follows, void (*kern)(P...), dim3 grid, int thread
     at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at.val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = &at;
-    cfg.numAttrs = follows && (int64_t)grid.x * grid.y * grid.z <= kChainCtas ? 1 : 0;
+    cfg.numAttrs = follows ? 1 : 0;
     return cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
 }
-__device__ __forceinline__ void chain_wait()
-{
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-}
+__device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 // Sets ctx->chain for a scope whose launches on s follow one another directly: no
 // profiling events between them, and no capture (its graph keeps full dependencies).
 struct ChainScope {

@@ -570,7 +570,6 @@ __global__ void __launch_bounds__(XYCfg<T, LB, RMAX>::THREADS)
     constexpr int b = C::b, bm = b - 1, NV = C::NV, NS = C::NS, HL = RMAX, LD = C::LD;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     T *s = reinterpret_cast<T *>(smem_raw);         // [NS][EY][LD], planes PL apart
-    chain_wait();
     __shared__ int nbs[(2 * kMaxWinNr + 2) * (2 * kMaxWinNr + 1)];
     const int o1 = at.items[2 * at.item], o2 = at.items[2 * at.item + 1];
     const bool pair = o2 >= 0;                      // uniform over the CTA
