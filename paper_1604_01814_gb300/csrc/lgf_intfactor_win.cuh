@@ -535,35 +535,62 @@ __global__ void __launch_bounds__(Cfg<T, LB, 2>::THREADS)
 // read per output.
 // 556 blocks of 16^3 (3 fields, RMAX 8): 38 -> 30 us; the 64-plate batch's launch
 // 712 -> 488 us.
-template <typename T, int LB, int RMAX>
+// FP64 is bound by its pipe (two lanes a clock and SM): what counts is that every SM
+// has work and that no warp is issued half empty.  So a CTA takes one z-plane (two
+// with blocks of 8) and 4 outputs per item, in items that fill whole warps.  With the
+// FP32 split, 8 blocks of 16^3 at windows 8, 12 and 16 were 16 CTAs: 31, 47 and 66 us (one
+// field), now 14, 17 and 22; 640 blocks of 32^3 at window 8 2517 -> 2390, 640 of 8^3 at
+// window 16 109 -> 93.  WIDE keeps 16 outputs per item where that is faster, as it holds the
+// window's inputs in registers: 640 blocks of 32^3 at window 16 2812 us against 3313, 640 of
+// 16^3 at window 12 324 against 353 and at 16 430 against 502 (see xy_wide).
+template <typename T, int LB, int RMAX, bool WIDE>
 struct XYCfg {
     static constexpr int b = 1 << LB, E = b + 2 * RMAX;
     static constexpr int EY1 = b + 2 * RMAX, EY = 2 * b + 2 * RMAX;   // staged rows: single, pair
     static constexpr int NV = 16 / (int)sizeof(T);
     static constexpr int LD = E + NV;                                // row pitch
-    static constexpr int V = b < 16 ? b : 16, GX = b / V;            // x outputs per thread, threads per row
-    static constexpr int VY = 8, GY = b / VY;                        // y outputs per thread
-    static constexpr int NS = 8 * EY * GX <= 256 ? 8 : 4 * EY * GX <= 256 ? 4 : 2 * EY * GX <= 256 ? 2 : 1;
-    static constexpr int THREADS = (NS * EY * GX + 31) / 32 * 32;
+    static constexpr bool F64 = sizeof(T) == 8, LOOP = F64;          // more x items than threads
+    static constexpr int V = !WIDE ? 4 : b < 16 ? b : 16, GX = b / V;   // x outputs per item, items per row
+    static constexpr int VY = !WIDE || (F64 && b == 32) ? 4 : 8, GY = b / VY;   // y outputs per item
+    static constexpr int NS = !WIDE ? (b < 16 ? 2 : 1)
+                            : F64 ? (b == 32 ? 1 : RMAX <= 12 ? 4 : 2)
+                            : 8 * EY * GX <= 256 ? 8 : 4 * EY * GX <= 256 ? 4 : 2 * EY * GX <= 256 ? 2 : 1;
+    static constexpr int THREADS = !WIDE ? 128
+                                 : F64 ? (b == 32 || RMAX == 16 ? 192 : 224)
+                                 : (NS * EY * GX + 31) / 32 * 32;
     static constexpr int RB = b * (int)sizeof(T);                    // bytes of a row of outputs
     static constexpr int SKEW = RB >= 128 ? 0 : (RB + 128 - EY * LD * (int)sizeof(T) % 128) % 128 / (int)sizeof(T);
     static constexpr int PL = EY * LD + SKEW;                        // plane pitch
     static constexpr size_t SMEM = sizeof(T) * (size_t)NS * PL;
-    static_assert(THREADS <= 256 && b % NS == 0 && SKEW % NV == 0, "one row item per thread, aligned planes");
+    static_assert(THREADS <= 256 && b % NS == 0 && SKEW % NV == 0, "aligned planes");
+    static_assert(32 % GX == 0, "the items of a row share a warp");
 };
 constexpr int kMaxWinNr = 2;   // neighbour blocks on a side: RMAX <= 16, b >= 8
+// Whether a launch over `items` blocks or pairs (times jobs and fields) takes the wide
+// form.  FP32: always.  FP64: blocks of 32 at window 16; blocks of 16 at windows 12 and 16
+// from 32 items on (64 blocks: 47.2 against 47.6 us and 57.5 against 66; 8 blocks: 47 against
+// 17 and 31 against 22).  At the other windows it is never faster.
+template <typename T, int LB, int RMAX>
+constexpr bool kXYEverWide = sizeof(T) == 4 || (LB == 5 && RMAX == 16) || (LB == 4 && RMAX >= 12);
+template <typename T, int LB, int RMAX>
+constexpr bool kXYEverNarrow = sizeof(T) == 8 && !(LB == 5 && RMAX == 16);
+template <typename T, int LB, int RMAX>
+constexpr bool xy_wide(int64_t items)
+{
+    return kXYEverWide<T, LB, RMAX> && (!kXYEverNarrow<T, LB, RMAX> || items >= 32);
+}
 
 // items: [n][2] output blocks (second -1 for a single block); nbr: for every
 // output block its (2nr+1)^2 xy neighbourhood of source blocks.
-template <typename T, int LB, int RMAX, class Tab = SepJobs<T>>
-__global__ void __launch_bounds__(XYCfg<T, LB, RMAX>::THREADS)
+template <typename T, int LB, int RMAX, bool WIDE, class Tab = SepJobs<T>>
+__global__ void __launch_bounds__(XYCfg<T, LB, RMAX, WIDE>::THREADS)
     k_sep_xy(const __grid_constant__ Tab jobs, const int *__restrict__ nbr_arg, const int *__restrict__ items_arg,
              int nr_arg)
 {
     const SepAt<T> at = sep_at(jobs, nbr_arg, items_arg, nr_arg);
     const SepJob<T> &J = *at.J;
     const int nr = at.nr;
-    using C = XYCfg<T, LB, RMAX>;
+    using C = XYCfg<T, LB, RMAX, WIDE>;
     using VT = typename Vec<T>::V;
     using CV = Col8<T>;
     using V8 = typename CV::V;
@@ -605,12 +632,12 @@ __global__ void __launch_bounds__(XYCfg<T, LB, RMAX>::THREADS)
     async::copies_done();
     __syncthreads();
     // ---- x stencil ----
-    {
+    auto x_item = [&](int it) {
         constexpr int V = C::V, NIN = V + 2 * RMAX;
         int zl, yr;
-        split(tid / C::GX, zl, yr);
-        const bool on = tid < NS * rows * C::GX;
-        T *row = s + (on ? zl * C::PL + yr * LD : 0) + (tid % C::GX) * V;
+        split(it / C::GX, zl, yr);
+        const bool on = it < NS * rows * C::GX;
+        T *row = s + (on ? zl * C::PL + yr * LD : 0) + (it % C::GX) * V;
         T in[NIN], acc[V];
         if (on) {
 #pragma unroll
@@ -621,7 +648,7 @@ __global__ void __launch_bounds__(XYCfg<T, LB, RMAX>::THREADS)
                 for (int e = 0; e < NV; ++e) in[i * NV + e] = vs[e];
             }
         }
-        if (C::GX > 1) __syncwarp();   // the row's other half is read before this one is overwritten
+        if (C::GX > 1) __syncwarp();   // the whole row is read before any of it is overwritten
         if (on) {
 #pragma unroll
             for (int v = 0; v < V; ++v) acc[v] = T(0);
@@ -642,6 +669,12 @@ __global__ void __launch_bounds__(XYCfg<T, LB, RMAX>::THREADS)
                 *reinterpret_cast<VT *>(row + v) = q;
             }
         }
+    };
+    if constexpr (C::LOOP) {
+#pragma unroll 1
+        for (int base = 0; base < NS * rows * C::GX; base += C::THREADS) x_item(base + tid);
+    } else {
+        x_item(tid);   // one item per thread
     }
     __syncthreads();
     // ---- y stencil: one 8-byte column, VY consecutive outputs per item ----
@@ -668,12 +701,12 @@ __global__ void __launch_bounds__(XYCfg<T, LB, RMAX>::THREADS)
     }
 }
 
-template <typename T, int LB, int RMAX>
-lgf_status launch_xy_m(lgf_ctx *ctx, int nitems, const SepJobs<T> &jobs, cudaStream_t s, const int *nbr,
-                       const int *items, int nr)
+template <typename T, int LB, int RMAX, bool WIDE>
+lgf_status launch_xy_form(lgf_ctx *ctx, int nitems, const SepJobs<T> &jobs, cudaStream_t s, const int *nbr,
+                          const int *items, int nr)
 {
-    using C = XYCfg<T, LB, RMAX>;
-    auto kern = k_sep_xy<T, LB, RMAX>;
+    using C = XYCfg<T, LB, RMAX, WIDE>;
+    auto kern = k_sep_xy<T, LB, RMAX, WIDE>;
     if (C::SMEM > 48 * 1024) {
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM);
         if (e != cudaSuccess) return cuda_fail(ctx, e, "cudaFuncSetAttribute");
@@ -681,6 +714,18 @@ lgf_status launch_xy_m(lgf_ctx *ctx, int nitems, const SepJobs<T> &jobs, cudaStr
     dim3 grid(nitems, C::b / C::NS, jobs.n * jobs.nf);
     kern<<<grid, C::THREADS, C::SMEM, s>>>(jobs, nbr, items, nr);
     return LGF_OK;
+}
+
+template <typename T, int LB, int RMAX>
+lgf_status launch_xy_m(lgf_ctx *ctx, int nitems, const SepJobs<T> &jobs, cudaStream_t s, const int *nbr,
+                       const int *items, int nr)
+{
+    const bool wide = xy_wide<T, LB, RMAX>((int64_t)nitems * jobs.n * jobs.nf);
+    if constexpr (kXYEverWide<T, LB, RMAX>)
+        if (wide) return launch_xy_form<T, LB, RMAX, true>(ctx, nitems, jobs, s, nbr, items, nr);
+    if constexpr (kXYEverNarrow<T, LB, RMAX>)
+        if (!wide) return launch_xy_form<T, LB, RMAX, false>(ctx, nitems, jobs, s, nbr, items, nr);
+    return fail(ctx, LGF_ECUDA, "intfactor: no form of the xy pass");
 }
 
 template <typename T, int LB>
@@ -767,11 +812,11 @@ lgf_status rag_send_sep(lgf_ctx *ctx, SepRagJob<T> *jobs, int n, Launch launch)
     return LGF_OK;
 }
 
-template <typename T, int LB, int RMAX>
-lgf_status launch_xy_rag_m(lgf_ctx *ctx, SepRagJob<T> *jobs, int n, cudaStream_t s)
+template <typename T, int LB, int RMAX, bool WIDE>
+lgf_status launch_xy_rag_form(lgf_ctx *ctx, SepRagJob<T> *jobs, int n, cudaStream_t s)
 {
-    using C = XYCfg<T, LB, RMAX>;
-    auto kern = k_sep_xy<T, LB, RMAX, SepRag<T>>;
+    using C = XYCfg<T, LB, RMAX, WIDE>;
+    auto kern = k_sep_xy<T, LB, RMAX, WIDE, SepRag<T>>;
     if (C::SMEM > 48 * 1024) {
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM);
         if (e != cudaSuccess) return cuda_fail(ctx, e, "cudaFuncSetAttribute");
@@ -779,6 +824,19 @@ lgf_status launch_xy_rag_m(lgf_ctx *ctx, SepRagJob<T> *jobs, int n, cudaStream_t
     return rag_send_sep<T>(ctx, jobs, n, [&](unsigned gx, const SepRag<T> &t) {
         kern<<<dim3(gx, C::b / C::NS, 1), C::THREADS, C::SMEM, s>>>(t, nullptr, nullptr, 0);
     });
+}
+
+template <typename T, int LB, int RMAX>
+lgf_status launch_xy_rag_m(lgf_ctx *ctx, SepRagJob<T> *jobs, int n, cudaStream_t s)
+{
+    int64_t items = 0;
+    for (int i = 0; i < n; ++i) items += (int64_t)jobs[i].nitems * jobs[i].nf;
+    const bool wide = xy_wide<T, LB, RMAX>(items);
+    if constexpr (kXYEverWide<T, LB, RMAX>)
+        if (wide) return launch_xy_rag_form<T, LB, RMAX, true>(ctx, jobs, n, s);
+    if constexpr (kXYEverNarrow<T, LB, RMAX>)
+        if (!wide) return launch_xy_rag_form<T, LB, RMAX, false>(ctx, jobs, n, s);
+    return fail(ctx, LGF_ECUDA, "intfactor: no form of the xy pass");
 }
 
 template <typename T, int LB, int RMAX>

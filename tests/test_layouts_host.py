@@ -1,0 +1,48 @@
+"""How the FP64 and long-line kernels split their work, from the constants they
+are compiled with (host programs over the kernel headers, no GPU needed).
+
+FP64 issues two lanes a clock and SM, so what it pays for is warps issued, full
+or not, and SMs without work; shared memory is paid in 128-byte wavefronts."""
+import os
+import shutil
+import subprocess
+
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+CSRC = os.path.join(ROOT, "paper_1604_01814_gb300", "csrc")
+NVCC = shutil.which("nvcc") or "/usr/local/cuda/bin/nvcc"
+
+
+def run(tmp_path, header, body):
+    """Lines of integers that `body` prints."""
+    if not os.path.exists(NVCC):
+        pytest.skip("no nvcc")
+    src, exe = tmp_path / "layout.cu", tmp_path / "layout"
+    src.write_text(f'#include <cstdio>\n#include "{header}"\nusing namespace lgf;\n{body}\n')
+    subprocess.run([NVCC, "-std=c++17", "--expt-relaxed-constexpr", "-gencode", "arch=compute_103a,code=sm_103a",
+                    "-I", os.path.join(ROOT, "include"), "-I", CSRC, "-o", str(exe), str(src)], check=True)
+    out = subprocess.run([str(exe)], check=True, capture_output=True, text=True).stdout
+    return [[int(v) for v in line.split()] for line in out.splitlines()]
+
+
+def test_fp64_xy_items_fill_warps_and_planes_spread(tmp_path):
+    """The x+y pass of small FP64 sets: every z-plane (two with blocks of 8) is a
+    CTA of its own, and the x and y items of a single block and of a pair are whole
+    warps; the wide form only where it is chosen, on larger sets."""
+    rows = run(tmp_path, "lgf_intfactor_win.cuh", r"""
+template <int LB, int R> void one() {
+    using C = win::XYCfg<double, LB, R, false>;
+    printf("%d %d %d %d %d %d %d %d %d %d\n", C::b, R, C::NS, C::EY1 * C::GX * C::NS, C::EY * C::GX * C::NS,
+           C::b * C::NS * C::GY, C::THREADS, (int)win::xy_wide<double, LB, R>(31), (int)win::xy_wide<double, LB, R>(32),
+           (int)win::xy_wide<float, LB, R>(1));
+}
+template <int LB> void all() { one<LB, 4>(); one<LB, 8>(); one<LB, 12>(); one<LB, 16>(); }
+int main() { all<3>(); all<4>(); all<5>(); }""")
+    assert len(rows) == 12
+    for b, R, ns, x1, x2, y1, threads, small, large, f32 in rows:
+        assert ns == (2 if b == 8 else 1)
+        assert x1 % 32 == x2 % 32 == y1 % 32 == 0 and threads % 32 == 0
+        assert f32 == 1
+        assert small == (b == 32 and R == 16)
+        assert large == (small or (b == 16 and R >= 12))
