@@ -366,10 +366,17 @@ struct ZCfg {
 // the staged k_sep_win.  Measured in FP32, staged over k_sep_z time: blocks of 16,
 // 1.03 to 1.6 from 8 to 3000 blocks and at every window; blocks of 32 (two runs along
 // z, so more of the window is fetched twice), window up to 8: 0.9 to 1.0 up to 125
-// blocks, 1.04 at 192, 1.15 at 375; windows 12 and 16: 0.75 to 1.02.  Equal in FP64, which
-// its arithmetic bounds.  Blocks of 8: a plane has too few columns for a CTA.
-template <int LB, int RMAX>
-constexpr bool z_march(int64_t blocks) { return LB == 4 || (LB == 5 && RMAX <= 8 && blocks >= 192); }
+// blocks, 1.04 at 192, 1.15 at 375; windows 12 and 16: 0.75 to 1.02.  FP64 (three fields):
+// blocks of 16 at windows 8 to 16 1.00 to 1.05, but 0.88 at window 4 (640 blocks: staged 128
+// us, k_sep_z 145), where the planes fetched twice outweigh the arithmetic; blocks of 32
+// 0.87 at window 4 (943 against 1086 us), equal at 8.  Blocks of 8: a plane has too few
+// columns for a CTA.
+template <typename T, int LB, int RMAX>
+constexpr bool z_march(int64_t blocks)
+{
+    if (sizeof(T) == 8) return LB == 4 && RMAX >= 8;
+    return LB == 4 || (LB == 5 && RMAX <= 8 && blocks >= 192);
+}
 template <typename T, int LB, int RMAX, class Tab = SepJobs<T>>
 __global__ void __launch_bounds__(ZCfg<T, LB>::THREADS)
     k_sep_z(const __grid_constant__ Tab jobs, const int *__restrict__ nbr_arg, int nr_arg)
@@ -771,7 +778,7 @@ lgf_status launch_m(lgf_ctx *ctx, int nout, const SepJobs<T> &jobs, cudaStream_t
     }
     if constexpr (AX == 2 && LB >= 4) {
         using Z = ZCfg<T, LB>;
-        if (z_march<LB, RMAX>((int64_t)nout * jobs.n * jobs.nf)) {
+        if (z_march<T, LB, RMAX>((int64_t)nout * jobs.n * jobs.nf)) {
             const cudaError_t e = chain_launch(ctx && ctx->chain, k_sep_z<T, LB, RMAX>, dim3(nout, Z::NY, jobs.n * jobs.nf),
                                                Z::THREADS, 0, s, jobs, nbr, nr);
             return e == cudaSuccess ? LGF_OK : cuda_fail(ctx, e, "intfactor z pass");
@@ -846,7 +853,7 @@ lgf_status launch_z_rag_m(lgf_ctx *ctx, SepRagJob<T> *jobs, int n, cudaStream_t 
         using Z = ZCfg<T, LB>;
         int64_t blocks = 0;
         for (int i = 0; i < n; ++i) blocks += (int64_t)jobs[i].nitems * jobs[i].nf;
-        if (z_march<LB, RMAX>(blocks))
+        if (z_march<T, LB, RMAX>(blocks))
             return rag_send_sep<T>(ctx, jobs, n, [&](unsigned gx, const SepRag<T> &t) {
                 k_sep_z<T, LB, RMAX, SepRag<T>><<<dim3(gx, Z::NY, 1), Z::THREADS, 0, s>>>(t, nullptr, 0);
             });

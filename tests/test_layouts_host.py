@@ -46,3 +46,18 @@ int main() { all<3>(); all<4>(); all<5>(); }""")
         assert f32 == 1
         assert small == (b == 32 and R == 16)
         assert large == (small or (b == 16 and R >= 12))
+
+
+def test_z_pass_choice(tmp_path):
+    """Which z pass: blocks of 16 stream in FP32, and in FP64 from window 8 on;
+    blocks of 32 stream in FP32 only, at windows 4 and 8, on large sets."""
+    rows = run(tmp_path, "lgf_intfactor_win.cuh", r"""
+template <int LB, int R> void one() {
+    printf("%d %d %d %d %d %d\n", 1 << LB, R, (int)win::z_march<float, LB, R>(1), (int)win::z_march<float, LB, R>(192),
+           (int)win::z_march<double, LB, R>(1), (int)win::z_march<double, LB, R>(100000));
+}
+template <int LB> void all() { one<LB, 4>(); one<LB, 8>(); one<LB, 12>(); one<LB, 16>(); }
+int main() { all<3>(); all<4>(); all<5>(); }""")
+    for b, R, few, many, few64, many64 in rows:
+        assert few == (b == 16) and many == (b == 16 or (b == 32 and R <= 8))
+        assert few64 == many64 == (b == 16 and R >= 8)
