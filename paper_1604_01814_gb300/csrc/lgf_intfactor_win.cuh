@@ -377,6 +377,7 @@ constexpr bool z_march(int64_t blocks)
     if (sizeof(T) == 8) return LB == 4 && RMAX >= 8;
     return LB == 4 || (LB == 5 && RMAX <= 8 && blocks >= 192);
 }
+constexpr int64_t kMarchAny = int64_t(1) << 62;   // more blocks than any launch has
 template <typename T, int LB, int RMAX, class Tab = SepJobs<T>>
 __global__ void __launch_bounds__(ZCfg<T, LB>::THREADS)
     k_sep_z(const __grid_constant__ Tab jobs, const int *__restrict__ nbr_arg, int nr_arg)
@@ -776,7 +777,7 @@ lgf_status launch_m(lgf_ctx *ctx, int nout, const SepJobs<T> &jobs, cudaStream_t
             return LGF_OK;
         }
     }
-    if constexpr (AX == 2 && LB >= 4) {
+    if constexpr (AX == 2 && z_march<T, LB, RMAX>(kMarchAny)) {
         using Z = ZCfg<T, LB>;
         if (z_march<T, LB, RMAX>((int64_t)nout * jobs.n * jobs.nf)) {
             const cudaError_t e = chain_launch(ctx && ctx->chain, k_sep_z<T, LB, RMAX>, dim3(nout, Z::NY, jobs.n * jobs.nf),
@@ -784,14 +785,17 @@ lgf_status launch_m(lgf_ctx *ctx, int nout, const SepJobs<T> &jobs, cudaStream_t
             return e == cudaSuccess ? LGF_OK : cuda_fail(ctx, e, "intfactor z pass");
         }
     }
-    auto kern = k_sep_win<T, LB, AX, RMAX>;
-    if (smem > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return cuda_fail(ctx, e, "cudaFuncSetAttribute");
+    if constexpr (AX != 2 || !z_march<T, LB, RMAX>(0)) {
+        auto kern = k_sep_win<T, LB, AX, RMAX>;
+        if (smem > 48 * 1024) {
+            cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            if (e != cudaSuccess) return cuda_fail(ctx, e, "cudaFuncSetAttribute");
+        }
+        dim3 grid(nout, b / C::NS, jobs.n * jobs.nf);
+        const cudaError_t e = chain_launch(ctx && ctx->chain, kern, grid, C::THREADS, smem, s, jobs, nbr, nr);
+        if (e != cudaSuccess) return cuda_fail(ctx, e, "intfactor pass");
     }
-    dim3 grid(nout, b / C::NS, jobs.n * jobs.nf);
-    const cudaError_t e = chain_launch(ctx && ctx->chain, kern, grid, C::THREADS, smem, s, jobs, nbr, nr);
-    return e == cudaSuccess ? LGF_OK : cuda_fail(ctx, e, "intfactor pass");
+    return LGF_OK;
 }
 
 // Ragged launches: every job field but cta0 set; sent in tables of
@@ -849,7 +853,7 @@ lgf_status launch_xy_rag_m(lgf_ctx *ctx, SepRagJob<T> *jobs, int n, cudaStream_t
 template <typename T, int LB, int RMAX>
 lgf_status launch_z_rag_m(lgf_ctx *ctx, SepRagJob<T> *jobs, int n, cudaStream_t s)
 {
-    if constexpr (LB >= 4) {
+    if constexpr (z_march<T, LB, RMAX>(kMarchAny)) {
         using Z = ZCfg<T, LB>;
         int64_t blocks = 0;
         for (int i = 0; i < n; ++i) blocks += (int64_t)jobs[i].nitems * jobs[i].nf;
@@ -858,17 +862,20 @@ lgf_status launch_z_rag_m(lgf_ctx *ctx, SepRagJob<T> *jobs, int n, cudaStream_t 
                 k_sep_z<T, LB, RMAX, SepRag<T>><<<dim3(gx, Z::NY, 1), Z::THREADS, 0, s>>>(t, nullptr, 0);
             });
     }
-    using C = Cfg<T, LB, 2>;
-    constexpr int b = 1 << LB, E = b + 2 * RMAX;
-    constexpr size_t smem = sizeof(T) * (size_t)C::NS * b * E;
-    auto kern = k_sep_win<T, LB, 2, RMAX, SepRag<T>>;
-    if (smem > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return cuda_fail(ctx, e, "cudaFuncSetAttribute");
+    if constexpr (!z_march<T, LB, RMAX>(0)) {
+        using C = Cfg<T, LB, 2>;
+        constexpr int b = 1 << LB, E = b + 2 * RMAX;
+        constexpr size_t smem = sizeof(T) * (size_t)C::NS * b * E;
+        auto kern = k_sep_win<T, LB, 2, RMAX, SepRag<T>>;
+        if (smem > 48 * 1024) {
+            cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            if (e != cudaSuccess) return cuda_fail(ctx, e, "cudaFuncSetAttribute");
+        }
+        return rag_send_sep<T>(ctx, jobs, n, [&](unsigned gx, const SepRag<T> &t) {
+            kern<<<dim3(gx, b / C::NS, 1), C::THREADS, smem, s>>>(t, nullptr, 0);
+        });
     }
-    return rag_send_sep<T>(ctx, jobs, n, [&](unsigned gx, const SepRag<T> &t) {
-        kern<<<dim3(gx, b / C::NS, 1), C::THREADS, smem, s>>>(t, nullptr, 0);
-    });
+    return LGF_OK;
 }
 
 template <typename T, int LB, int AX>
