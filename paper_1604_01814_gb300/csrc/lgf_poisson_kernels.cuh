@@ -625,24 +625,35 @@ constexpr int congruent(int v, int c) { return v + (((c - v) % 16) + 16) % 16; }
 template <typename T, int ML>
 struct RowLay {
     using P = Plan<ML>;
-    // threads per line: 16 to 24 values each (a masked last round where TPC
-    // does not divide the first stage's groups); TPC is a multiple of R0 in the
-    // three-stage plans
-    static constexpr int TPC = ML <= 32 ? 4
+    // threads per line: 8 to 48 values each; TPC is a multiple of R0 in the
+    // three-stage plans.  Where TPC does not divide the first stage's groups, the
+    // lanes past them are idle in the last round: free in FP32, but FP64 issues a
+    // warp over 16 cycles whatever its lanes do, so it takes the counts that leave
+    // none idle (x forward, 3 fields of 96 x 96 lines: length 192 145 -> 130 us, 160 162 -> 129; 512x512
+    // lines of length 32, half a warp a CTA before, 279 -> 145)
+    static constexpr bool F64 = sizeof(T) == 8;
+    static constexpr int TPC = F64 && (ML == 80 || ML == 160) ? 10
+                             : F64 && (ML == 96 || ML == 192) ? 12
+                             : F64 && ML == 640 ? 16
+                             : ML <= 32 ? 4
                              : ML <= 160 ? 8
                              : ML == 320 ? 20
                              : ML <= 384 ? 16
                              : ML <= 768 || ML == 1280 ? 32
                              : ML == 2048 || ML == 4096 ? 128
                                          : 64;
-    // lines per CTA: 8 up to length 768 (32 for the shortest lines, which would
-    // leave a CTA of one warp), 4 above, so that several CTAs of an SM overlap
+    // lines per CTA: 8 up to length 768 and at 1280 (32 for the shortest lines in
+    // FP32, which would leave a CTA of one warp), 4 above, or 2 or 1 where 4 lines do not
+    // fit, so that several CTAs of an SM overlap
     // their loads, stages and stores and a small box still fills the GPU: 16 lines at
     // length 256 took the 128^3 box's batch from 99.7 to 105.3 us, 8 lines
-    // at length 1024 the wake's x forward from 648 to 804 us
+    // at length 1024 the wake's x forward from 648 to 804 us.  FP64: 4 at 64 and 128,
+    // so that every SM has lines (below), 16 at 160 for whole warps
     static constexpr int SIZE = int(sizeof(Cx<T>));
     static constexpr bool fit(int l) { return (ML * (l + 1) + 64 + ML) * SIZE <= 112 * 1024; }
-    static constexpr int LPC = sizeof(T) == 8 && ML <= 128 ? 4   // (FP64: every SM needs lines)
+    static constexpr int LPC = F64 && (ML == 64 || ML == 128) ? 4
+                             : F64 && ML == 160 ? 16
+                             : F64 && ML < 128 ? 8
                              : TPC == 4 ? 32
                              : (ML <= 768 || ML == 1280) && fit(8) ? 8
                              : fit(4) ? 4 : ML * SIZE <= 48 * 1024 ? 2 : 1;

@@ -61,3 +61,37 @@ int main() { all<3>(); all<4>(); all<5>(); }""")
     for b, R, few, many, few64, many64 in rows:
         assert few == (b == 16) and many == (b == 16 or (b == 32 and R <= 8))
         assert few64 == many64 == (b == 16 and R >= 8)
+
+
+SIZES = (32, 64, 80, 96, 128, 160, 192, 256, 320, 384, 512, 640, 768, 1024, 1280, 1536, 2048, 2560, 3072, 4096)
+
+
+def _warps(active):
+    """Warps with an active lane, of a list of lane flags."""
+    return sum(any(active[i:i + 32]) for i in range(0, len(active), 32))
+
+
+def _idle(threads, lane, groups, tpc):
+    """Warps issued over warps' worth of groups: thread i of `threads` is lane(i)
+    of its line's tpc, and takes groups lane, lane + tpc, ..."""
+    issued = sum(_warps([lane(i) + r < groups for i in range(threads)]) for r in range(0, groups, tpc))
+    lines = threads // tpc
+    return issued * 32 / (lines * groups)
+
+
+def test_fp64_x_passes_leave_no_lanes_idle(tmp_path):
+    rows = run(tmp_path, "lgf_poisson_kernels.cuh", r"""
+template <int M> void one() {
+    using P = pk::Plan<M>; using L = pk::RowLay<double, M>;
+    printf("%d %d %d %d %d\n", M, L::THREADS, L::TPC, P::G0, P::GL);
+}
+template <int... M> void all() { (one<M>(), ...); }
+int main() { all<""" + ", ".join(map(str, SIZES)) + ">(); }")
+    assert len(rows) == len(SIZES)
+    for M, threads, tpc, g0, gl in rows:
+        lpc = threads // tpc
+        first = _idle(threads, lambda i: i % tpc, g0, tpc)      # lanes along the groups of a line
+        last = _idle(threads, lambda i: i // lpc, gl, tpc)      # lanes along the lines
+        assert first <= 1.2 and last <= 1.0, (M, first, last)
+        if M != 80:
+            assert first == 1.0, (M, first)
