@@ -1059,7 +1059,9 @@ struct ColCfg {
     // columns, not how many CTAs share one.  With 32 columns a CTA the 32^3 box (length
     // 64) had 33 CTAs in the y passes and 66 in z: 72.6 us, now 51.2; the FP64 sphere
     // Poisson apply 3623 -> 3548 us
-    static constexpr int W0 = sizeof(T) == 8 ? 8 : TPC <= 8 ? 32 : TPC <= 20 ? 16 : 8;
+    // At length 160 the 10 groups of the first stage are 2.5 warps of 8 columns, half
+    // a warp idle in the dearer stage: 16 columns (z pass of 96x96x80 points, 3 fields: 890 -> 814 us)
+    static constexpr int W0 = sizeof(T) == 8 ? (ML == 160 ? 16 : 8) : TPC <= 8 ? 32 : TPC <= 20 ? 16 : 8;
     static constexpr int WMAX = int(98304 / (sizeof(Cx<T>) * ML)) < 1 ? 1 : int(98304 / (sizeof(Cx<T>) * ML));
     static constexpr int W = W0 < WMAX ? W0 : WMAX;
     static constexpr size_t SMEM = sizeof(Cx<T>) * (((size_t)ML) * (W + 1));

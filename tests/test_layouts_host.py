@@ -95,3 +95,20 @@ int main() { all<""" + ", ".join(map(str, SIZES)) + ">(); }")
         assert first <= 1.2 and last <= 1.0, (M, first, last)
         if M != 80:
             assert first == 1.0, (M, first)
+
+
+def test_fp64_column_passes_leave_few_lanes_idle(tmp_path):
+    """Columns side by side in a warp; the idle part weighted by the stages' radix
+    (five flops per point and binary digit)."""
+    import math
+    rows = run(tmp_path, "lgf_poisson_kernels.cuh", r"""
+template <int M> void one() {
+    using P = pk::Plan<M>; using C = pk::ColCfg<double, M>;
+    printf("%d %d %d %d %d %d %d\n", M, C::W, P::TPC, P::G0, P::GL, P::R0, P::RL);
+}
+template <int... M> void all() { (one<M>(), ...); }
+int main() { all<""" + ", ".join(map(str, SIZES)) + ">(); }")
+    for M, w, tpc, g0, gl, r0, rl in rows:
+        cost = [math.log2(r0), math.log2(rl)]
+        idle = [_idle(w * tpc, lambda i: i // w, g, tpc) for g in (g0, gl)]
+        assert sum(c * i for c, i in zip(cost, idle)) / sum(cost) < 1.1, (M, idle)
