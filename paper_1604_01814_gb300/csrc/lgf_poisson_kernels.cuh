@@ -141,19 +141,30 @@ __device__ __forceinline__ void dit_group(Cx<T> *a, int j, const Cx<T> *tw)
 }
 
 // Middle stage (three-stage plans): shared memory to shared memory.  The
-// threads of a line split as TS sub-problems times TJ groups, so that every
+// threads of a line split as TJ groups times TS sub-problems, so that every
 // group's address is the thread's own plus a constant.
+template <int ML>
+struct MidSplit {
+    using P = Plan<ML>;
+    // Consecutive threads take consecutive groups, which are neighbours in shared
+    // memory; sub-problems are a multiple of all banks apart.  With the
+    // sub-problems along the threads the 11 threads of a warp at length 4096 (three
+    // columns) met on the same banks: z pass of 64x64x2048 points 450 us (373 before that
+    // split, 325 now), y passes of 32x1024x512 264 and 217 (249 and 207; 251 and 202 now);
+    // at 512 (1024x512x512, 12 fields) z 7.2 -> 6.3 ms.
+    static constexpr int TJ = cgcd(P::TPC, P::RL), TS = P::TPC / TJ;
+    static_assert(P::NST == 2 || (P::R0 % TS == 0 && P::RL % TJ == 0), "whole groups per thread");
+};
 template <int ML, int DIR, typename T, class Addr>
 __device__ __forceinline__ void middle_stage(Cx<T> *s, const Addr &ad, int line, int t, const Cx<T> *tw)
 {
     using P = Plan<ML>;
     if constexpr (P::NST == 3) {
         constexpr int N = P::N1, R = P::R1, NP = N / R;
-        constexpr int TS = cgcd(P::TPC, P::R0), TJ = P::TPC / TS;
-        static_assert(NP % TJ == 0, "whole groups per thread");
-        const int j0 = t / TS;
+        constexpr int TS = MidSplit<ML>::TS, TJ = MidSplit<ML>::TJ;
+        const int j0 = t % TJ;
         const Cx<T> *tw1 = tw + P::TW1 + j0;
-        const int o = (t % TS) * N + j0;
+        const int o = (t / TJ) * N + j0;
 #pragma unroll
         for (int sub = 0; sub < P::R0; sub += TS) {
 #pragma unroll

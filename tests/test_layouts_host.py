@@ -112,3 +112,29 @@ int main() { all<""" + ", ".join(map(str, SIZES)) + ">(); }")
         cost = [math.log2(r0), math.log2(rl)]
         idle = [_idle(w * tpc, lambda i: i // w, g, tpc) for g in (g0, gl)]
         assert sum(c * i for c, i in zip(cost, idle)) / sum(cost) < 1.1, (M, idle)
+
+
+def test_middle_stage_wavefronts(tmp_path):
+    """Shared-memory wavefronts of the column passes' middle stage (FP32, element m
+    of column w at m W + w, 16 lanes of 8 bytes): at most a third above the least."""
+    rows = run(tmp_path, "lgf_poisson_kernels.cuh", r"""
+template <int M> void one() {
+    using P = pk::Plan<M>; using C = pk::ColCfg<float, M>;
+    if constexpr (P::NST == 3)
+        printf("%d %d %d %d %d %d\n", M, C::W, P::TPC, pk::MidSplit<M>::TJ, pk::MidSplit<M>::TS, P::N1);
+}
+template <int... M> void all() { (one<M>(), ...); }
+int main() { all<""" + ", ".join(map(str, SIZES)) + ">(); }")
+    assert [r[0] for r in rows] == [m for m in SIZES if m >= 384]
+    for M, w, tpc, tj, ts, n1 in rows:
+        assert tj * ts == tpc
+        waves = least = 0
+        for half in range(0, w * tpc, 16):
+            words = set()
+            for i in range(half, min(half + 16, w * tpc)):
+                t = i // w
+                words.add(((t // tj) * n1 + t % tj) * w + i % w)
+            banks = [v % 16 for v in words]
+            waves += max(banks.count(k) for k in set(banks))
+            least += 1
+        assert waves <= 4 / 3 * least, (M, waves, least)
