@@ -67,10 +67,11 @@ struct PoissonChoice {
     int bump[3] = {0, 0, 0}; // transform length: the bump-th supported length above the smallest valid one
     int zvar = 0;
     int fuse = 0;            // fused y+x inverse (FP32, where instantiated; the tuner's alternative)
+    int zwin = 1;            // z: the shifted window where x or y is shifted and it is shorter
     bool operator==(const PoissonChoice &o) const
     {
         return shift[0] == o.shift[0] && shift[1] == o.shift[1] && bump[0] == o.bump[0] && bump[1] == o.bump[1] &&
-               bump[2] == o.bump[2] && zvar == o.zvar && fuse == o.fuse;
+               bump[2] == o.bump[2] && zvar == o.zvar && fuse == o.fuse && zwin == o.zwin;
     }
 };
 
@@ -358,6 +359,9 @@ lgf_status poisson_plan(lgf_ctx *ctx, const lgf_blockset *src, const lgf_blockse
 bool poisson_geometry(const PoissonPlan &pl, const PoissonChoice &ch, PoissonGeom *g, int64_t *A, int64_t *B);
 // Default choice: the shifted window on x and y where it is shorter.
 PoissonChoice poisson_default_choice(const PoissonPlan &pl, bool allow_shift);
+// A persisted choice (lgf_tune.h).
+struct TuneChoiceText;
+PoissonChoice tune_choice(const TuneChoiceText &t);
 // Apply a choice to the plan (geometry and scratch sizes).
 void poisson_set_choice(PoissonPlan *pl, const PoissonChoice &ch);
 lgf_status poisson_spectrum(lgf_ctx *ctx, const PoissonGeom &pg, double alpha, Spectrum **out, cudaStream_t s);

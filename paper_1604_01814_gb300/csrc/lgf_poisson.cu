@@ -121,7 +121,7 @@ bool poisson_geometry(const PoissonPlan &pl, const PoissonChoice &ch, PoissonGeo
         g.nbs[d] = pl.shi[d] - pl.slo[d] + 1;
         g.nbt[d] = pl.thi[d] - pl.tlo[d] + 1;
         bool shift = d < 2 && ch.shift[d];
-        if (d == 2 && (ch.shift[0] || ch.shift[1])) {
+        if (d == 2 && ch.zwin && (ch.shift[0] || ch.shift[1])) {
             // z follows x and y: shifted where that is shorter.  Its spectrum has all kz
             // (twice the values of one shifted in x or y, which is complex
             // already; an even one would grow from a real half, so z alone stays even)

@@ -56,20 +56,22 @@ TuneChoiceText to_text(const PoissonChoice &c)
     for (int d = 0; d < 3; ++d) t.bump[d] = c.bump[d];
     t.zvar = c.zvar;
     t.fuse = c.fuse;
+    t.zwin = c.zwin;
     return t;
 }
 
-PoissonChoice from_text(const TuneChoiceText &t)
+}  // namespace
+
+PoissonChoice tune_choice(const TuneChoiceText &t)
 {
     PoissonChoice c;
     for (int d = 0; d < 2; ++d) c.shift[d] = t.shift[d];
     for (int d = 0; d < 3; ++d) c.bump[d] = t.bump[d];
     c.zvar = t.zvar;
     c.fuse = t.fuse;
+    c.zwin = t.zwin;
     return c;
 }
-
-}  // namespace
 
 lgf_status tune_poisson(lgf_ctx *ctx, PoissonPlan *pl, int nf, double kalpha, cudaStream_t s)
 {
@@ -80,8 +82,8 @@ lgf_status tune_poisson(lgf_ctx *ctx, PoissonPlan *pl, int nf, double kalpha, cu
         TuneChoiceText t;
         PoissonGeom g = pl->g;
         int64_t A, B;
-        if (tune_parse_plan_value(it->second, &t) && poisson_geometry(*pl, from_text(t), &g, &A, &B)) {
-            poisson_set_choice(pl, from_text(t));
+        if (tune_parse_plan_value(it->second, &t) && poisson_geometry(*pl, tune_choice(t), &g, &A, &B)) {
+            poisson_set_choice(pl, tune_choice(t));
             pl->tuned_nf = nf;
             ++ctx->tune_plans_cached;
             return LGF_OK;

@@ -6,7 +6,10 @@
 // comments.  A Poisson plan's key names everything its timing depends on
 // (precision, block edge, block extents of source and target and their
 // offset, field count) and its value the choice:
-//   P f32 b16 s4,2,4 t67,4,4 o-1,-1,0 nf3 -> x1 y1 bx0 by0 bz0 z0
+//   P f32 b16 s4,2,4 t67,4,4 o-1,-1,0 nf3 -> x1 y1 bx0 by0 bz0 z0 f0 w1
+// (w1: z takes the shifted window where x or y does and it is shorter.  Choices
+// written before z had that window end earlier and were timed with z even, which
+// they keep.)
 // A batch's key is a hash of its shape (block sets, operations, field
 // counts) and its value the branch count:
 //   B f32 9f3a... -> nb4
@@ -24,6 +27,7 @@ struct TuneChoiceText {
     int bump[3] = {0, 0, 0};
     int zvar = 0;
     int fuse = 0;
+    int zwin = 0;
 };
 
 inline std::string tune_plan_key(bool f64, int b, const int nbs[3], const int nbt[3], const int off[3], int nf)
@@ -39,6 +43,7 @@ inline std::string tune_plan_value(const TuneChoiceText &c)
     std::ostringstream o;
     o << "x" << c.shift[0] << " y" << c.shift[1] << " bx" << c.bump[0] << " by" << c.bump[1] << " bz" << c.bump[2]
       << " z" << c.zvar << " f" << c.fuse;
+    if (c.zwin) o << " w" << c.zwin;
     return o.str();
 }
 
@@ -48,10 +53,10 @@ inline bool tune_parse_plan_value(const std::string &v, TuneChoiceText *c)
     TuneChoiceText t;
     // (files written before the fused inverse existed end after the z field:
     // the inverse then stays apart, the default)
-    const int nread = std::sscanf(v.c_str(), "x%d y%d bx%d by%d bz%d z%d f%d", &t.shift[0], &t.shift[1], &t.bump[0],
-                                  &t.bump[1], &t.bump[2], &t.zvar, &t.fuse);
-    if (nread != 6 && nread != 7) return false;
-    if (t.fuse < 0 || t.fuse > 1) return false;
+    const int nread = std::sscanf(v.c_str(), "x%d y%d bx%d by%d bz%d z%d f%d w%d", &t.shift[0], &t.shift[1], &t.bump[0],
+                                  &t.bump[1], &t.bump[2], &t.zvar, &t.fuse, &t.zwin);
+    if (nread < 6) return false;
+    if (t.fuse < 0 || t.fuse > 1 || t.zwin < 0 || t.zwin > 1) return false;
     for (int d = 0; d < 2; ++d)
         if (t.shift[d] < 0 || t.shift[d] > 1) return false;
     for (int d = 0; d < 3; ++d)

@@ -33,8 +33,9 @@ def problem(M, yshift, mirror=False):
     return li.Problem("z", b, np.array(src, np.int32), np.array(tgt, np.int32), f)
 
 
-def library_geometry(tmp_path, problems):
-    """(M_x, M_y, M_z, shifted x, y, z) of the plans that the library makes by default."""
+def library_geometry(tmp_path, problems, choice=""):
+    """(M_x, M_y, M_z, shifted x, y, z) of the plans that the library makes by default, or
+    for a choice as a tuning file states it."""
     nvcc = shutil.which("nvcc") or "/usr/local/cuda/bin/nvcc"
     csrc = os.path.join(ROOT, "paper_1604_01814_gb300", "csrc")
     objs = glob.glob(os.path.join(ROOT, "_build", "*.cu.o"))
@@ -48,8 +49,11 @@ def library_geometry(tmp_path, problems):
 #include <algorithm>
 #include <cstdio>
 #include "lgf_internal.cuh"
-int main()
+#include "lgf_tune.h"
+int main(int argc, char **argv)
 {
+    lgf::TuneChoiceText text;
+    if (argc > 1 && !lgf::tune_parse_plan_value(argv[1], &text)) return 3;
     int b, ns, nt;
     while (scanf("%d %d %d", &b, &ns, &nt) == 3) {
         lgf::PoissonPlan p;
@@ -65,7 +69,8 @@ int main()
             }
         lgf::PoissonGeom g{};
         int64_t A, B;
-        if (!lgf::poisson_geometry(p, lgf::poisson_default_choice(p, true), &g, &A, &B)) return 2;
+        if (!lgf::poisson_geometry(p, argc > 1 ? lgf::tune_choice(text) : lgf::poisson_default_choice(p, true), &g, &A, &B))
+            return 2;
         printf("%d %d %d %d %d %d\n", g.M[0], g.M[1], g.M[2], g.xasym, g.yasym, g.zasym);
     }
 }
@@ -75,8 +80,21 @@ int main()
                     os.path.join(ROOT, "include"), "-I", csrc, "-o", str(exe), str(main), *objs], check=True)
     text = "".join(f"{p.b} {len(p.src)} {len(p.tgt)}\n" + "\n".join(" ".join(map(str, c)) for c in np.concatenate([p.src, p.tgt])) +
                    "\n" for p in problems)
-    out = subprocess.run([str(exe)], input=text, check=True, capture_output=True, text=True).stdout
-    return [tuple(map(int, line.split())) for line in out.splitlines()]
+    run = lambda *args: [tuple(map(int, line.split())) for line in
+                         subprocess.run([str(exe), *args], input=text, check=True, capture_output=True, text=True).stdout.splitlines()]
+    return run(choice) if choice else run()
+
+
+def test_choices_of_older_files_keep_z_even(tmp_path):
+    """A choice written before z had a shifted window was timed with z even and names
+    that geometry still; one written now ends with w1."""
+    probs = [problem(64, 1), problem(320, 0)]
+    new = library_geometry(tmp_path, probs, "x1 y0 bx0 by0 bz0 z0 f0 w1")
+    assert [g[2] for g in new] == [64, 320] and all(g[5] for g in new)
+    for old in ("x1 y0 bx0 by0 bz0 z0", "x1 y0 bx0 by0 bz0 z0 f0"):
+        got = library_geometry(tmp_path, probs, old)
+        assert [g[2] for g in got] == [128, 640] and not any(g[5] for g in got)
+    assert library_geometry(tmp_path, probs[1:], "x1 y0 bx0 by0 bz1 z0")[0][2] == 768
 
 
 def test_default_geometry(tmp_path):
