@@ -204,13 +204,13 @@ PoissonPlan::~PoissonPlan()
 
 namespace {
 
-// Entry i of a length's table: exp(-2 pi i exps[i] / M).
-__global__ void k_twiddles(int M, const int *__restrict__ exps, void *out, int dbl)
+// Entry i of a length's table: exp(-2 pi i e_i / M), in the order of its stage plan.
+__global__ void k_twiddles(int M, int R0, int R1, void *out, int dbl)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= M) return;
     double s, c;
-    sincospi(-2.0 * exps[i] / M, &s, &c);
+    sincospi(-2.0 * pk::twiddle_exponent(i, M, R0, R1) / M, &s, &c);
     if (dbl) {
         ((Cx<double> *)out)[i] = {c, s};
     } else {
@@ -218,18 +218,15 @@ __global__ void k_twiddles(int M, const int *__restrict__ exps, void *out, int d
     }
 }
 
-// The table's exponents in the order of the length's stage plan.
+// The first two radices of a length's stage plan.
 template <int ML>
-lgf_status fill_exponents(std::vector<int> *e)
+lgf_status radices_m(int *R0, int *R1)
 {
-    for (int i = 0; i < ML; ++i) (*e)[i] = pk::twiddle_exponent<ML>(i);
+    *R0 = pk::Plan<ML>::R0;
+    *R1 = pk::Plan<ML>::R1;
     return LGF_OK;
 }
-lgf_status twiddle_exponents(lgf_ctx *ctx, int M, std::vector<int> *e)
-{
-    e->assign(M, 0);
-    LGF_DISPATCH_ML(M, fill_exponents<LM>(e));
-}
+lgf_status plan_radices(lgf_ctx *ctx, int M, int *R0, int *R1) { LGF_DISPATCH_ML(M, radices_m<LM>(R0, R1)); }
 
 // Spectrum of a shifted window: the complex forward transform at
 // kx <= Mx/2, ky < nky (My/2 + 1 when the window is even in y, My when it
@@ -389,23 +386,16 @@ const void *twiddles(lgf_ctx *ctx, int M, bool dbl, lgf_status *st)
     auto &tab = dbl ? ctx->tw64 : ctx->tw32;
     auto it = tab.find(M);
     if (it != tab.end()) return it->second;
-    std::vector<int> exps;
-    if ((*st = twiddle_exponents(ctx, M, &exps)) != LGF_OK) return nullptr;
+    int R0 = 0, R1 = 0;
+    if ((*st = plan_radices(ctx, M, &R0, &R1)) != LGF_OK) return nullptr;
     void *p = nullptr;
-    int *ed = nullptr;
     cudaError_t e = cudaMalloc(&p, (size_t)M * (dbl ? 16 : 8));
-    if (e == cudaSuccess) e = cudaMalloc(&ed, (size_t)M * sizeof(int));
     if (e != cudaSuccess) {
-        cudaFree(p);
         *st = fail(ctx, LGF_ENOMEM, "twiddle table allocation failed");
         return nullptr;
     }
-    e = cudaMemcpy(ed, exps.data(), (size_t)M * sizeof(int), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) {
-        k_twiddles<<<(M + 255) / 256, 256>>>(M, ed, p, dbl ? 1 : 0);
-        e = cudaDeviceSynchronize();
-    }
-    cudaFree(ed);
+    k_twiddles<<<(M + 255) / 256, 256>>>(M, R0, R1, p, dbl ? 1 : 0);
+    e = cudaDeviceSynchronize();
     if (e != cudaSuccess) {
         cudaFree(p);
         *st = cuda_fail(ctx, e, "twiddle kernel");

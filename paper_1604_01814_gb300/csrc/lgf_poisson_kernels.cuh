@@ -85,13 +85,12 @@ __device__ __forceinline__ int pos_of(int k)
 // Exponent e of entry i of a length's twiddle table (the entry is
 // exp(-2 pi i e / M)): the first stage's w_M^{j q} at (q - 1) G0 + j, then the
 // middle stage's w_{N1}^{j q} = w_M^{j q R0} at TW1 + (q - 1) RL + j; 0 past them.
-template <int ML>
-int twiddle_exponent(int i)
+__host__ __device__ inline int twiddle_exponent(int i, int M, int R0, int R1)
 {
-    using P = Plan<ML>;
-    if (i < P::TW1) return (i % P::G0) * (i / P::G0 + 1);
-    i -= P::TW1;
-    return P::NST == 3 && i < (P::R1 - 1) * P::RL ? (i % P::RL) * (i / P::RL + 1) * P::R0 : 0;
+    const int G0 = M / R0, RL = G0 / R1, TW1 = (R0 - 1) * G0;
+    if (i < TW1) return (i % G0) * (i / G0 + 1);
+    i -= TW1;
+    return i < (R1 - 1) * RL ? (i % RL) * (i / RL + 1) * R0 : 0;   // (none with R1 = 1)
 }
 
 template <int ML>

@@ -138,3 +138,25 @@ int main() { all<""" + ", ".join(map(str, SIZES)) + ">(); }")
             waves += max(banks.count(k) for k in set(banks))
             least += 1
         assert waves <= 4 / 3 * least, (M, waves, least)
+
+
+def test_twiddle_tables_take_one_allocation_and_no_upload(tmp_path):
+    """Entry i of a length's table in the order of its stages (the first use of a
+    length forms it on the device): w_M^{j q} at (q - 1) G0 + j, then w_{N1}^{j q}."""
+    rows = run(tmp_path, "lgf_poisson_kernels.cuh", r"""
+template <int M> void one() {
+    using P = pk::Plan<M>;
+    printf("%d %d %d", M, P::R0, P::R1);
+    for (int i = 0; i < M; ++i) printf(" %d", pk::twiddle_exponent(i, M, P::R0, P::R1));
+    printf("\n");
+}
+template <int... M> void all() { (one<M>(), ...); }
+int main() { all<""" + ", ".join(map(str, SIZES)) + ">(); }")
+    for M, r0, r1, *e in rows:
+        g0, rl = M // r0, M // r0 // r1
+        want = [j * q for q in range(1, r0) for j in range(g0)] + [j * q * r0 for q in range(1, r1) for j in range(rl)]
+        assert e == want + [0] * (M - len(want)), M
+    text = open(os.path.join(CSRC, "lgf_poisson.cu")).read()
+    body = text[text.index("const void *twiddles("):]
+    body = body[:body.index("\n}\n")]
+    assert body.count("cudaMalloc(") == 1 and "cudaMemcpy" not in body
