@@ -401,7 +401,7 @@ LGF_API lgf_status lgf_ctx_stats(lgf_ctx *ctx, lgf_stats *out);
 
 /* Set the cache bounds: max_plans (per plan kind, >= 1; default 256 Poisson
    and integrating-factor plans, 64 curl and IB plans), max_spectra (>= 1,
-   default 32) and max_graphs (>= 0, default 8; 0 runs every batch with direct
+   default 128) and max_graphs (>= 0, default 8; 0 runs every batch with direct
    launches).  -1 keeps a bound.  Lowering a bound takes effect at the next
    insertion.  Changing max_graphs drops the cached graphs.
    Errors: LGF_EINVAL. */

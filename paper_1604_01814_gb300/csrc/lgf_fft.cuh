@@ -31,7 +31,10 @@ template <typename R>
 __device__ __forceinline__ Cx<R> cmul(Cx<R> a, Cx<R> b) { return {a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x}; }
 // The same sum and difference of the power-of-two butterflies: in FP32 one packed
 // instruction for both components (a difference as a + (-1) b, rounded once, the
-// same value).  The passes are bound by issue slots, and a packed add takes one where
+// same value).  Where a scalar e + (x c - y s) may be contracted into two fused
+// operations, the packed add keeps its own rounding: results moved by 6e-8 to 7e-8 of the
+// largest, their errors against 64 bits by rounding only (128^3 box 1.39e-7 -> 1.42e-7).
+// The passes are bound by issue slots, and a packed add takes one where
 // two scalar adds take two; the FP32 pipes' rate is the same.  At length 256 (16 x
 // 16) the z pass of the sphere set went from 85 to 65 us.  The butterflies around
 // the 3- and 5-point ones stay scalar (packed, the y inverse at length 192 went from 35

@@ -124,7 +124,11 @@ bool poisson_geometry(const PoissonPlan &pl, const PoissonChoice &ch, PoissonGeo
         if (d == 2 && ch.zwin && (ch.shift[0] || ch.shift[1])) {
             // z follows x and y: shifted where that is shorter.  Its spectrum has all kz
             // (twice the values of one shifted in x or y, which is complex
-            // already; an even one would grow from a real half, so z alone stays even)
+            // already; an even one would grow from a real half, so z alone stays even).
+            // The larger spectrum weighs most with one field, and it pays there too: 17 body
+            // and flow pairs of 16^3 blocks (6x6x6 to 40x12x12), z even over shifted time, 0.99
+            // to 1.38 in FP32 (three fields 1.00 to 1.43), 1.00 to 1.42 in FP64; below 25 us,
+            // where launches bound the apply, 0.96 to 1.01
             const int Ms = fft_size_bumped(g.Ls[2] + g.Lt[2] - 1, ch.bump[2]);
             shift = 2 * g.Ls[2] <= Ms && Ms <= kMaxFft && Ms < fft_size_bumped((int)std::min<int64_t>(2 * L - 1, 2 * kMaxFft), ch.bump[2]);
             g.zasym = shift;
@@ -547,10 +551,10 @@ lgf_status poisson_spectrum(lgf_ctx *ctx, const PoissonGeom &pg, double alpha, S
     double *box = nullptr;
     Cx<double> *A = nullptr, *B = nullptr;
     void *spec = nullptr;
-    // layouts: even x and y: reals [kz][ky <= My/2][kx]; shifted x: complex,
-    // same shape; shifted y: complex [kz][ky < My][kx] (no symmetry in ky)
+    // layouts [kz][ky][kx]: all axes even: reals at kz <= Mz/2, ky <= My/2; shifted x:
+    // complex, same shape; shifted y or z: complex, all ky or kz (no symmetry there)
     const int nky = pg.yasym ? M[1] : M[1] / 2 + 1;
-    const int nkz = pg.zasym ? M[2] : M[2] / 2 + 1;   // and in kz where z is shifted
+    const int nkz = pg.zasym ? M[2] : M[2] / 2 + 1;
     const bool cplx = pg.xasym || pg.yasym || pg.zasym;
     const size_t spec_elems = (size_t)pg.ld * nky * nkz * (cplx ? 2 : 1);
     const size_t esz = ctx->prec == LGF_F64 ? 8 : 4;

@@ -34,8 +34,10 @@ namespace pk {
 // either padding, m + (m >> A) + (m >> B), or a swizzle of the low four
 // bits, m ^ (((m >> A) ^ (m >> B)) & 15) (a permutation inside each aligned
 // run of 16).  The (kind, A, B) per length came from a model of those
-// accesses that counts shared-memory wavefronts per half-warp; it cuts them
-// from 2.3x to 1.5x the conflict-free count on average.  B = 0: no second term.
+// accesses that counts shared-memory wavefronts per half-warp; it cut them
+// from 2.3x to 1.5x the conflict-free count on average, with three stages (or a
+// radix of 20) at 80, 96, 160, 192 and 320, whose plans have two stages now.  B = 0: no
+// second term.
 template <int ML>
 struct RowAddr {
     static constexpr int KIND = ML == 512 || ML == 768 || ML == 1280 || ML == 1536 || ML == 2560 || ML == 3072 ||

@@ -31,7 +31,8 @@ constexpr int cgcd(int a, int b) { return b == 0 ? a : cgcd(b, a % b); }
 // divisor of the stages' group counts, so that every thread owns a whole number of
 // groups in every stage; the two-stage plans have one group per thread in the
 // longer stage, and the threads past the shorter stage's groups (whole warps,
-// as lanes run along columns) sit it out.
+// as lanes run along columns) sit it out.  (Length 32 keeps the divisor, 4: its threads own
+// whole groups of both stages.)
 // Lengths 96, 192 and 320 had three stages (4 x 2 x 12, 4 x 4 x 12, 4 x 4 x 20), 80 and
 // 160 a radix of 20: with two stages half the shared-memory passes and barriers go,
 // and more of the butterflies are packed.  z pass at length 320 (refresh of 556 blocks)

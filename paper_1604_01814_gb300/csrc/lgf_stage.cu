@@ -9,7 +9,8 @@
 //   (G q)_k(n)  = [q(n) - q(n - e_k)] / dx               cells -> faces
 // and G^dagger = -Dbar.  Both read the block itself and, where the shift
 // leaves it, the neighbour block of a CurlPlan (dir +1 for Dbar, -1 for G);
-// values outside the input block set are zero.  One thread per output cell.
+// values outside the input block set are zero.  A thread makes 16 bytes of a row of
+// outputs.
 #include <algorithm>
 #include <cstring>
 

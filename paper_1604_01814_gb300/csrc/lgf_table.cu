@@ -217,11 +217,9 @@ __global__ void k_lookup(const double *table, int R, const int32_t *off, int64_t
     out[i] = lgf_value(table, R, off[3 * i], off[3 * i + 1], off[3 * i + 2]);
 }
 
-// Even circular embedding of G_L on an Mx x My x Mz box:
-// box[z][y][x] = G_L(min(x, Mx-x), min(y, My-y), min(z, Mz-z)).
-// Circular embedding of G_L on an Mx x My x Mz box: even along z
-// (h[m] = G_L(min(m, M - m))); along x and y the window h[m] = G_L(m + c) for
-// m < P and G_L(m - M + c) above (c = 0, P = M/2 is the even one).
+// Circular embedding of G_L on an Mx x My x Mz box: along each axis the window
+// h[m] = G_L(m + c) for m < P and G_L(m - M + c) above; c = 0 and P = M/2 is the even
+// one, h[m] = G_L(min(m, M - m)).
 __global__ void k_window(const double *table, int R, int Mx, int My, int Mz, int xc, int xP, int yc, int yP, int zc,
                          int zP, double *box)
 {
