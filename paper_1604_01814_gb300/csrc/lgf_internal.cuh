@@ -273,8 +273,9 @@ namespace lgf {
 // free, and stayed there: E(0.75) of 8 FP64 blocks of 32 took 171 us (76 unchained, 74
 // now), the FP64 box of 96x32x32 275 us (190, 179), 16x128x128 in FP32 57 (40, 31),
 // 32x32x384 56 (44, 33).  Against plain launches it hides the launch and those fetches:
-// 24^3 apply 26.6 -> 20.2 us, sphere Poisson apply 147 -> 138, sphere stage 766 -> 742; over
-// 1000 calls from 16^3 to 10^8 points none is slower, so there is no limit on the grid.
+// 24^3 apply 26.5 -> 21 us, sphere Poisson apply 148 -> 137, sphere stage 769 -> 737; of 760
+// calls of 512 to 6e7 points none above 20 us (where the host bounds them) is more than
+// 2 % slower, so there is no limit on the grid.
 template <class... P, class... A>
 cudaError_t chain_launch(bool follows, void (*kern)(P...), dim3 grid, int threads, size_t smem, cudaStream_t s, A... args)
 {

@@ -361,6 +361,11 @@ struct ZCfg {
     static constexpr int LANES = b * b / Col8<T>::N;   // columns of a block
     static constexpr int THREADS = LANES < 128 ? LANES : 128;
     static constexpr int NY = (LANES / THREADS) * (b / V);   // grid.y: slices of the plane, runs along z
+    // Blocks of 32: up to 96 registers, all loads in flight (the compiler's own 64 for
+    // resident CTAs: E at window 8 of 640 blocks, 3 fields, 269 -> 254 us, 261 with the 56
+    // that it took beside an early release of dependents).  Blocks of 16: its own choice (35
+    // against 35 us for 640 blocks, 245 against 252 for 2880 at window 16).
+    static constexpr int OCC = LB == 5 && sizeof(T) == 4 ? 1 : 0;
 };
 // Whether a launch over `blocks` output blocks (times jobs and fields) takes k_sep_z or
 // the staged k_sep_win.  Measured in FP32, staged over k_sep_z time: blocks of 16,
@@ -379,7 +384,7 @@ constexpr bool z_march(int64_t blocks)
 }
 constexpr int64_t kMarchAny = int64_t(1) << 62;   // more blocks than any launch has
 template <typename T, int LB, int RMAX, class Tab = SepJobs<T>>
-__global__ void __launch_bounds__(ZCfg<T, LB>::THREADS)
+__global__ void __launch_bounds__(ZCfg<T, LB>::THREADS, ZCfg<T, LB>::OCC)
     k_sep_z(const __grid_constant__ Tab jobs, const int *__restrict__ nbr_arg, int nr_arg)
 {
     using C = ZCfg<T, LB>;
